@@ -13,6 +13,7 @@
 
 #include "eis.h"
 #include "eis_bsgs.cuh"
+#include "eis_cubic.cuh"
 #include "eis_internal.h"
 #include "eis_kernels.h"
 
@@ -70,6 +71,7 @@ struct eis_ctx {
     int occ_persistent = 1;
     int occ_record = 1;                     // resident CTAs/SM of k_walk_record
     int occ_bsgs = 1;                       // ... and of k_bsgs
+    int occ_cubic = 1;                      // ... and of k_cubic
     std::vector<eis_tune_row> tune;         // per-decade lane-search settings (empty: none)
     eis_stats last{};
 };
@@ -93,7 +95,8 @@ struct eis_plan {
     Tile *d_tiles = nullptr;
     uint32_t *d_sqfree = nullptr, *d_flags = nullptr;
     uint32_t *d_tile_pop = nullptr, *d_tile_off = nullptr, *d_surv = nullptr;
-    uint32_t *d_ctr = nullptr;  // [0] survivors, [1] queue head
+    uint32_t *d_ctr = nullptr;  // [0] survivors, [1] queue head, [2] handed to k_giant,
+                                // [3] its head, [4] head of k_cubic
     int *d_status = nullptr;
     unsigned long long *d_counts = nullptr;  // [2 s] #E, [2 s + 1] #D
     unsigned long long *d_steps = nullptr;   // [0] baby, [1] giant, [2] deferred
@@ -119,6 +122,12 @@ struct eis_plan {
     uint32_t *d_bctr = nullptr;  // [0] walk head [1] records [3] search head
                                  // [4] fallbacks [5] fallback walk head
     std::vector<cudaEvent_t> bev;  // per round: start, after the walk, end
+    // cubic forms (eis_cubic.cuh): jobs over the segments where they pay
+    std::vector<CubicJob> cubic;
+    uint32_t cubic_units = 0, cubic_grid = 0;
+    CubicJob *d_cubic = nullptr;
+    uint32_t *d_field = nullptr;   // [a cubic field of discriminant d], null with a log output
+    uint8_t *d_segfield = nullptr; // per segment: d_field holds its candidates
     uint64_t bytes = 0;
     uint32_t walk_grid = 0;
     int launches = 0;
@@ -256,6 +265,32 @@ static constexpr uint32_t kBsgsMaxCycles = 1u << 20;  // giant cycles per d befo
 // search's table pool is not worth allocating for them).
 static constexpr uint64_t kBsgsMinCands = (uint64_t)1 << 18;
 
+// Cubic forms are used while the step limit is at least its default, above
+// any half period below 2^44: a lower limit asks that every walk be held to
+// it, and so that every d be walked.
+static constexpr int64_t kCubicMinStepLimit = (int64_t)1 << 26;
+// ... and in plans where they save at least this much (thread instructions;
+// about 15 us of the whole GPU, the cost of their launches).
+static constexpr double kCubicMinGain = 4e8;
+
+// What the cubic forms save on a segment, in thread instructions (negative:
+// they cost more).  A walk takes about 0.067 sqrt(d) steps of 13.3
+// instructions (with the lane search, about 18.9 d^(1/4) steps' worth); the
+// forms decide 0.87 of the square-free d (with a log output only those in E,
+// about 0.29).  The enumeration looks at about 0.135 d^(3/4) triples for
+// kind 0 and 0.057 d^(3/4) for kind 1, whatever the window's width (counted
+// at 10^9 .. 2^44), each about 200 instructions.
+static double cubic_gain(const Seg &s, bool search, bool with_log, bool primes) {
+    if (s.ncand == 0) return -1.0;
+    const double d = (double)(s.d0 + 8 * (s.ncand - 1));
+    double steps = 0.067 * std::sqrt(d);
+    if (search) steps = std::min(steps, 18.9 * std::sqrt(std::sqrt(d)));
+    const double density = primes ? 4.0 / std::log(d) : 0.81;
+    const double walk = (double)s.ncand * density * steps * 13.3 * (with_log ? 0.29 : 0.87);
+    const double forms = 200.0 * std::pow(d, 0.75) * (with_log ? 0.135 : 0.192);
+    return 0.8 * walk - forms;
+}
+
 static void record(cudaEvent_t ev, cudaStream_t s, bool capturing) {
     if (capturing)
         cudaEventRecordWithFlags(ev, s, cudaEventRecordExternal);
@@ -271,7 +306,7 @@ static int plan_enqueue(eis_plan *p, cudaStream_t s, bool capturing) {
     int launches = 0;
     record(p->ev[0], s, capturing);
     EIS_CK(cudaMemsetAsync(p->d_flags, 0, p->nwords * 4, s));
-    EIS_CK(cudaMemsetAsync(p->d_ctr, 0, 4 * sizeof(uint32_t), s));
+    EIS_CK(cudaMemsetAsync(p->d_ctr, 0, 8 * sizeof(uint32_t), s));
     EIS_CK(cudaMemsetAsync(p->d_status, 0, sizeof(int), s));
     EIS_CK(cudaMemsetAsync(p->d_counts, 0, 2 * nseg * sizeof(unsigned long long) + 8, s));
     EIS_CK(cudaMemsetAsync(p->d_steps, 0, 4 * sizeof(unsigned long long), s));
@@ -282,15 +317,28 @@ static int plan_enqueue(eis_plan *p, cudaStream_t s, bool capturing) {
                                        p->d_tile_pop, p->primes_only);
         ++launches;
         if (p->mode == EIS_MODE_PERSISTENT) {
+            const bool cubic = !p->cubic.empty();
+            if (cubic) {
+                if (p->d_field) EIS_CK(cudaMemsetAsync(p->d_field, 0, p->nwords * 4, s));
+                k_cubic<<<p->cubic_grid, 256, 0, s>>>(p->d_cubic, (uint32_t)p->cubic.size(),
+                                                      p->cubic_units, p->d_ctr + 4, p->d_flags,
+                                                      p->d_field);
+                k_select<<<ntiles, 256, 0, s>>>(p->d_tiles, p->d_sqfree, p->d_flags, p->d_field,
+                                                p->d_segfield, p->d_glog, p->d_tile_pop);
+                launches += 2;
+            }
             k_scan_tiles<<<1, 1024, 0, s>>>(p->d_tile_pop, p->d_tile_off, ntiles, p->d_ctr);
-            k_compact<<<ntiles, 256, 0, s>>>(p->d_tiles, p->d_sqfree, p->d_tile_off, p->d_surv);
+            k_compact<<<ntiles, 256, 0, s>>>(p->d_tiles, p->d_sqfree, p->d_tile_off, p->d_surv,
+                                             cubic ? p->d_flags : nullptr, p->d_field,
+                                             p->d_segfield);
             launches += 2;
             record(p->ev[1], s, capturing);
             if (p->bsgs) {
                 const uint32_t C = p->bsgs_chunk;
                 for (uint32_t r = 0; r < p->bsgs_rounds; ++r) {
                     const uint32_t q_lo = r * C;
-                    const uint32_t q_hi = (uint32_t)std::min<uint64_t>((uint64_t)q_lo + C, 0xffffffffull);
+                    // the last round takes all that is left: past C records a d walks on
+                    const uint32_t q_hi = r + 1 == p->bsgs_rounds ? 0xffffffffu : q_lo + C;
                     record(p->bev[3 * r], s, capturing);
                     EIS_CK(cudaMemsetAsync(p->d_bctr, 0, 8 * sizeof(uint32_t), s));
                     k_walk_record<<<p->bsgs_grid_a, 256, 0, s>>>(
@@ -373,7 +421,8 @@ static void plan_free(eis_plan *p) {
     }
     void *bufs[] = {p->d_segs, p->d_tiles, p->d_sqfree, p->d_flags, p->d_tile_pop, p->d_tile_off,
                     p->d_surv, p->d_ctr, p->d_status, p->d_counts, p->d_steps, p->d_glog,
-                    p->d_defer, p->d_cls, p->d_recs, p->d_pool, p->d_fb, p->d_bctr};
+                    p->d_defer, p->d_cls, p->d_recs, p->d_pool, p->d_fb, p->d_bctr,
+                    p->d_cubic, p->d_field, p->d_segfield};
     for (void *b : bufs)
         if (b) cudaFree(b);
     if (p->ctx) ctx_release(p->ctx, p->bytes);
@@ -451,7 +500,7 @@ static int plan_build(eis_ctx *c, const uint64_t *lo, const uint64_t *hi, size_t
     EIS_ALLOC(p->d_tile_pop, ntiles * 4);
     EIS_ALLOC(p->d_tile_off, ntiles * 4);
     if (mode == EIS_MODE_PERSISTENT) EIS_ALLOC(p->d_surv, p->total_cand * 4);
-    EIS_ALLOC(p->d_ctr, 4 * sizeof(uint32_t));
+    EIS_ALLOC(p->d_ctr, 8 * sizeof(uint32_t));
     EIS_ALLOC(p->d_status, sizeof(int));
     EIS_ALLOC(p->d_counts, 2 * nseg * sizeof(unsigned long long) + 8);
     EIS_ALLOC(p->d_steps, 4 * sizeof(unsigned long long));
@@ -477,6 +526,45 @@ static int plan_build(eis_ctx *c, const uint64_t *lo, const uint64_t *hi, size_t
         p->tt.tau[0] = 1.39f / (float)c->mark_every;
         any_search = p->tt.nbaby[0] > 0;
     }
+    // cubic forms for the segments where they cost less than the walks they
+    // save; `left` is about what the queue will hold (all of a plain segment,
+    // at most 0.15 of a candidate's share where the forms decide: measured
+    // 0.09 to 0.11; with a log output all but the flagged)
+    uint64_t left = 0;
+    std::vector<uint8_t> segfield(nseg, 0);
+    uint64_t field_bytes = 0;
+    if (mode == EIS_MODE_PERSISTENT && c->step_limit >= kCubicMinStepLimit) {
+        double saved = 0;
+        for (size_t si = 0; si < nseg; ++si) {
+            const double gain = cubic_gain(p->segs[si], any_search, with_log, p->primes_only);
+            segfield[si] = gain > 0;
+            saved += std::max(0.0, gain);
+        }
+        if (saved < kCubicMinGain) std::fill(segfield.begin(), segfield.end(), 0);
+        uint64_t units = 0;
+        for (size_t si = 0; si < nseg; ++si) {
+            if (!segfield[si]) continue;
+            for (uint32_t kind = 0; kind < (with_log ? 1u : 2u); ++kind) {
+                CubicJob j{};
+                j.d0 = p->segs[si].d0;
+                j.ncand = p->segs[si].ncand;
+                j.bit0 = p->segs[si].cand0;
+                j.kind = kind;
+                cubic_job_bounds(j);
+                j.unit0 = (uint32_t)units;
+                units += cubic_units(j);
+                p->cubic.push_back(j);
+            }
+        }
+        if (units > 0xf0000000ull) p->cubic.clear();
+        p->cubic_units = (uint32_t)units;
+        p->cubic_grid = (uint32_t)std::min<uint64_t>((uint64_t)c->sm_count * c->occ_cubic, (units + 7) / 8);
+        if (!p->cubic.empty())
+            field_bytes = p->cubic.size() * sizeof(CubicJob) + nseg + 32 + (with_log ? 0 : p->nwords * 4);
+    }
+    for (size_t si = 0; si < nseg; ++si)
+        left += p->cubic.empty() || !segfield[si] || with_log ? p->segs[si].ncand
+                                                               : p->segs[si].ncand * 15 / 100 + 64;
     if (mode == EIS_MODE_PERSISTENT && any_search && p->total_cand >= kBsgsMinCands) {
         // lane-per-d search: survivors in rounds of C queue positions; the
         // pool holds one table region per resident lane plus one per d a
@@ -487,16 +575,17 @@ static int plan_build(eis_ctx *c, const uint64_t *lo, const uint64_t *hi, size_t
         const uint64_t per_d = kBsgsRegionBytes + sizeof(DRecord) + 4;
         const uint64_t used = c->in_use.load();
         const uint64_t cached = pool_cached_bytes(c);  // reclaimable
-        const uint64_t left = c->budget + cached > used ? c->budget + cached - used : 0;
-        const uint64_t fit = left / per_d > lanes + 64 ? left / per_d - lanes - 64 : 0;
-        uint64_t C = std::min<uint64_t>((uint64_t)c->bsgs_chunk, (p->total_cand + 31) / 32 * 32);
+        const uint64_t room = c->budget + cached > used + field_bytes ? c->budget + cached - used - field_bytes : 0;
+        const uint64_t fit = room / per_d > lanes + 64 ? room / per_d - lanes - 64 : 0;
+        const uint64_t queue = (left + 31) / 32 * 32;
+        uint64_t C = std::min<uint64_t>((uint64_t)c->bsgs_chunk, queue);
         C = std::min<uint64_t>(C, fit / 32 * 32);
-        if (C >= ((uint64_t)1 << 16) || C >= (p->total_cand + 31) / 32 * 32) {
+        if (C >= ((uint64_t)1 << 16) || C >= queue) {
             p->bsgs = 1;
             p->bsgs_walk_cap = (uint32_t)c->bsgs_walk_cap;
             p->bsgs_window = (uint32_t)(c->bsgs_window > 0 ? c->bsgs_window : c->bsgs_walk_cap);
             p->bsgs_chunk = (uint32_t)C;
-            p->bsgs_rounds = (uint32_t)((p->total_cand + C - 1) / C);
+            p->bsgs_rounds = (uint32_t)((left + C - 1) / C);
             p->bsgs_grid_a = (uint32_t)(c->sm_count * c->occ_record);
             p->bsgs_grid_b = (uint32_t)(c->sm_count * c->occ_bsgs);
             const uint64_t pool_need = (lanes + C) * kBsgsRegionBytes;
@@ -531,6 +620,19 @@ static int plan_build(eis_ctx *c, const uint64_t *lo, const uint64_t *hi, size_t
             occ = 1;
         }
         p->giant_grid = (uint32_t)(c->sm_count * std::max(1, occ));
+    }
+    if (!p->cubic.empty()) {
+        // without room for them the plan walks every d
+        if (plan_alloc(p, (void **)&p->d_cubic, p->cubic.size() * sizeof(CubicJob)) != EIS_OK ||
+            plan_alloc(p, (void **)&p->d_segfield, nseg) != EIS_OK ||
+            (!with_log && plan_alloc(p, (void **)&p->d_field, p->nwords * 4) != EIS_OK)) {
+            p->cubic.clear();
+        } else if (cudaMemcpy(p->d_cubic, p->cubic.data(), p->cubic.size() * sizeof(CubicJob),
+                              cudaMemcpyHostToDevice) != cudaSuccess ||
+                   cudaMemcpy(p->d_segfield, segfield.data(), nseg, cudaMemcpyHostToDevice) != cudaSuccess) {
+            plan_free(p);
+            return EIS_EDEVICE;
+        }
     }
 #undef EIS_ALLOC
     for (auto &e : p->ev) {
@@ -833,6 +935,9 @@ int eis_create(eis_ctx **out, int device, uint64_t mem_budget_bytes) {
                                                       128, 0) != cudaSuccess)
         occ = 1;
     c->occ_bsgs = std::max(1, occ);
+    occ = 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_cubic, 256, 0) != cudaSuccess) occ = 1;
+    c->occ_cubic = std::max(1, occ);
     cudaGetLastError();
     *out = c;
     return EIS_OK;
@@ -1304,7 +1409,7 @@ int eis_classify_range_u8(eis_ctx *c, uint64_t lo, uint64_t hi, uint8_t *codes_o
     uint64_t d0;
     const uint64_t ntot = num_candidates(lo, hi, &d0);
     eis_stats acc{};
-    int rc = run_chunks(c, lo, hi, 1, s, &acc, [&](eis_plan *p, uint64_t off) -> int {
+    int rc = run_chunks(c, lo, hi, 0, s, &acc, [&](eis_plan *p, uint64_t off) -> int {
         const uint64_t n = std::min<uint64_t>(p->total_cand, ntot - off);
         if (n == 0) return EIS_OK;
         uint8_t *tmp = out_on_device ? codes_out + off : nullptr;

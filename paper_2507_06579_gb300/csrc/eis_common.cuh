@@ -332,6 +332,12 @@ __device__ __forceinline__ uint64_t cand_to_d(const Seg *__restrict__ segs, uint
     return segs[lo].d0 + 8 * (cand - segs[lo].cand0);
 }
 
+// Candidates of a word left to the walk: square-free, not flagged, and with a
+// cubic field of discriminant d (`field`, all ones where that is not known).
+__device__ __forceinline__ uint32_t left_word(uint32_t sq, uint32_t flags, uint32_t field) {
+    return sq & ~flags & field;
+}
+
 // Block-wide sum of one value per thread (valid in thread 0).
 __device__ __forceinline__ uint32_t block_sum(uint32_t v, uint32_t *red) {
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(kFull, v, o);

@@ -6,6 +6,7 @@
 
 #include "eis_bsgs.cuh"
 #include "eis_common.cuh"
+#include "eis_cubic.cuh"
 
 namespace eis {
 
@@ -14,7 +15,13 @@ __global__ void k_sieve(const Tile *tiles, const Seg *segs, const uint32_t *prim
 __global__ void k_scan_tiles(const uint32_t *tile_pop, uint32_t *tile_off, uint32_t ntiles,
                              uint32_t *total);
 __global__ void k_compact(const Tile *tiles, const uint32_t *sqfree, const uint32_t *tile_off,
-                          uint32_t *surv);
+                          uint32_t *surv, const uint32_t *flags, const uint32_t *field,
+                          const uint8_t *seg_field);
+__global__ void k_cubic(const CubicJob *jobs, uint32_t njobs, uint32_t nunits, uint32_t *next_ptr,
+                        uint32_t *bits0, uint32_t *bits1);
+__global__ void k_select(const Tile *tiles, const uint32_t *sqfree, uint32_t *flags,
+                         const uint32_t *field, const uint8_t *seg_field, uint8_t *glog,
+                         uint32_t *tile_pop);
 __global__ void k_count(const Tile *tiles, const uint32_t *flags, const uint32_t *sqfree,
                         unsigned long long *counts, const uint8_t *glog, unsigned long long *cls);
 __global__ void k_expand_codes(const uint32_t *flags, const uint32_t *sqfree, uint64_t ncand,

@@ -205,7 +205,8 @@ bool launch_batch(eis_server *s, Slot &sl) {
         k_sieve<<<nt, 256, 0, st>>>(sl.d_tiles, sl.d_segs, cv.d_primes, cv.nprimes, sl.d_sqfree,
                                     sl.d_tile_pop, 0);
         k_scan_tiles<<<1, 1024, 0, st>>>(sl.d_tile_pop, sl.d_tile_off, nt, sl.d_ctr);
-        k_compact<<<nt, 256, 0, st>>>(sl.d_tiles, sl.d_sqfree, sl.d_tile_off, sl.d_surv);
+        k_compact<<<nt, 256, 0, st>>>(sl.d_tiles, sl.d_sqfree, sl.d_tile_off, sl.d_surv, nullptr,
+                                      nullptr, nullptr);
         k_walk_persistent<<<s->grid, 256, 0, st>>>(sl.d_segs, nseg, sl.d_surv, sl.d_ctr,
                                                    sl.d_ctr + 1, sl.d_flags, nullptr, sl.d_steps,
                                                    sl.d_status, s->step_limit, s->defer_after,

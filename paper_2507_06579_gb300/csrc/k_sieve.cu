@@ -138,19 +138,25 @@ __global__ void __launch_bounds__(1024) k_scan_tiles(const uint32_t *__restrict_
 // words' popcounts places each word's survivors in a shared-memory stage,
 // and the block copies the stage to the queue with consecutive threads
 // writing consecutive entries, so the queue is written in whole lines.
+// flags (or null): after k_select, only what the cubic forms left undecided.
 __global__ void __launch_bounds__(256) k_compact(const Tile *__restrict__ tiles,
                                                  const uint32_t *__restrict__ sqfree,
                                                  const uint32_t *__restrict__ tile_off,
-                                                 uint32_t *__restrict__ surv) {
+                                                 uint32_t *__restrict__ surv,
+                                                 const uint32_t *__restrict__ flags,
+                                                 const uint32_t *__restrict__ field,
+                                                 const uint8_t *__restrict__ seg_field) {
     __shared__ uint32_t red[32];
     __shared__ uint32_t stage[256 * 32];  // one chunk: at most 8192 survivors
     const Tile t = tiles[blockIdx.x];
     const uint32_t nw = (t.ncand + 31) >> 5;
     const uint64_t wbase = t.cand0 >> 5;
     uint32_t out = tile_off[blockIdx.x];
+    const bool use = field && seg_field[t.seg];
     for (uint32_t c0 = 0; c0 < nw; c0 += 256) {
         const uint32_t w = c0 + threadIdx.x;
         uint32_t x = (w < nw) ? sqfree[wbase + w] : 0u;
+        if (flags && x) x = left_word(x, flags[wbase + w], use ? field[wbase + w] : kFull);
         uint32_t tot;
         uint32_t o = block_excl_scan((uint32_t)__popc(x), red, &tot);
         const uint32_t cbase = (uint32_t)(t.cand0 + 32u * w);
