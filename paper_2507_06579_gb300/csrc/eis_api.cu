@@ -49,6 +49,7 @@ struct eis_ctx {
     std::vector<uint32_t> primes;  // host copy of the odd primes of d_primes
     int *d_single = nullptr;  // [0] result, [1] steps, [2] status
     unsigned char *d_query = nullptr;  // K3 single query: u64 d, i8 out, int status, u64 acc[2], u32 next
+    QueryOut *h_query = nullptr;       // k_query's answer: pinned host memory the device writes
     // A lane-search table pool kept from a freed plan for the next one (its
     // bytes stay charged to in_use): freeing and mapping tens of GB per plan
     // cost milliseconds in every eis_classify_range / eis_count_range call.
@@ -255,6 +256,16 @@ static void giant_params(uint64_t d, int64_t forced, int &nbaby, int &log2n) {
     nbaby = n;
     log2n = 2;
     while ((1 << log2n) < 4 * n) ++log2n;
+}
+
+// Baby-step count of a single query (k_query): 256 lanes of giant steps of
+// 1.5 N steps each should reach past most periods (about 0.13 sqrt(d) steps)
+// in one round.  Mean call in us for N = 256 / 512 / 1024: 74 / 76 / 85 near
+// 10^12, 86 / 85 / 95 near 4e12, 109 / 101 / 112 near 2^44 (p99 there 241 /
+// 158 / 143).
+static void query_params(uint64_t d, int64_t forced, int &nbaby, int &log2n) {
+    if (forced <= 0) forced = d < 4000000000000ull ? 512 : 1024;
+    giant_params(d, forced, nbaby, log2n);
 }
 
 static constexpr int kGiantMaxLog2 = 14;  // 128 KB table per warp at most
@@ -913,7 +924,13 @@ int eis_create(eis_ctx **out, int device, uint64_t mem_budget_bytes) {
         eis_destroy(c);
         return EIS_ENOMEM;
     }
-    if (cudaFuncSetAttribute(k_giant, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    if (cudaHostAlloc(&c->h_query, sizeof(QueryOut), cudaHostAllocMapped) != cudaSuccess) {
+        eis_destroy(c);
+        return EIS_ENOMEM;
+    }
+    if (cudaFuncSetAttribute(k_query, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)((8u << kGiantMaxLog2) + 16 * (4096 + 2))) != cudaSuccess ||
+        cudaFuncSetAttribute(k_giant, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)(8u << kGiantMaxLog2)) != cudaSuccess) {
         eis_destroy(c);
         return EIS_EDEVICE;
@@ -950,6 +967,7 @@ int eis_destroy(eis_ctx *c) {
     if (c->d_primes) cudaFree(c->d_primes);
     if (c->d_single) cudaFree(c->d_single);
     if (c->d_query) cudaFree(c->d_query);
+    if (c->h_query) cudaFreeHost(c->h_query);
     if (c->d_sqtab) cudaFree(c->d_sqtab);
     if (c->pool_cache) cudaFree(c->pool_cache);
     if (c->stream) cudaStreamDestroy(c->stream);
@@ -1464,23 +1482,41 @@ int eis_is_eisenstein(eis_ctx *c, uint64_t d, int *result_out) {
     std::memset(&c->last, 0, sizeof(c->last));
     c->last.candidates = 1;
     int res = 0;  // 0: not in D, else 1 + log eps_d
+    // only odd primes with p^2 <= d can divide d: scan those, on as many
+    // blocks as they fill (at most two per SM)
+    uint64_t r = (uint64_t)std::sqrt((double)d);
+    while (r * r > d) --r;
+    while ((r + 1) * (r + 1) <= d) ++r;
+    const uint32_t np = (uint32_t)(std::upper_bound(c->primes.begin(), c->primes.end(),
+                                                    (uint32_t)std::min<uint64_t>(r, UINT32_MAX)) -
+                                   c->primes.begin());
+    const uint32_t blocks = std::max<uint32_t>(1u, std::min<uint32_t>((np + 255) / 256,
+                                                                      (uint32_t)c->sm_count * 2));
+    if (c->mode == EIS_MODE_PERSISTENT && c->giant_compose == EIS_COMPOSE_TEXTBOOK) {
+        // one launch: a block searches, the others test for square factors
+        int nbaby, log2n;
+        query_params(d, c->giant_stride, nbaby, log2n);
+        volatile QueryOut *h = c->h_query;
+        h->result = 0;
+        h->square = h->baby = h->giant = 0;
+        k_query<<<1 + blocks, kQueryThreads, ((size_t)8 << log2n) + 16 * (nbaby + 2), c->stream>>>(
+            d, c->d_sqtab, np, c->h_query, nbaby, log2n, kGiantMaxRounds * 32 / kQueryThreads);
+        EIS_CK(cudaGetLastError());
+        EIS_CK(cudaStreamSynchronize(c->stream));
+        if (h->square) return EIS_ENOTD;
+        if (h->result <= 0) return EIS_ESTEPS;
+        c->last.baby_steps = h->baby;
+        c->last.giant_steps = h->giant;
+        c->last.in_D = 1;
+        c->last.in_E = (h->result == 1);
+        *result_out = (h->result == 1) ? 1 : 0;
+        return EIS_OK;
+    }
     // square-free test by the whole GPU (d_query[40], 0 = square-free)
     unsigned char *q = c->d_query;  // [0] d, [8] out, [12] status, [16] acc[2], [32] next, [40] flag
     uint32_t *sq_flag = reinterpret_cast<uint32_t *>(q + 40);
     EIS_CK(cudaMemsetAsync(q, 0, 64, c->stream));
-    {
-        // only odd primes with p^2 <= d can divide d: scan those, on as many
-        // blocks as they fill (at most two per SM)
-        uint64_t r = (uint64_t)std::sqrt((double)d);
-        while (r * r > d) --r;
-        while ((r + 1) * (r + 1) <= d) ++r;
-        const uint32_t np = (uint32_t)(std::upper_bound(c->primes.begin(), c->primes.end(),
-                                                        (uint32_t)std::min<uint64_t>(r, UINT32_MAX)) -
-                                       c->primes.begin());
-        const uint32_t blocks = std::max<uint32_t>(1u, std::min<uint32_t>((np + 255) / 256,
-                                                                          (uint32_t)c->sm_count * 2));
-        k_sqfree_one<<<blocks, 256, 0, c->stream>>>(d, c->d_sqtab, np, sq_flag);
-    }
+    k_sqfree_one<<<blocks, 256, 0, c->stream>>>(d, c->d_sqtab, np, sq_flag);
     EIS_CK(cudaGetLastError());
     if (c->mode == EIS_MODE_PLAIN) {
         // one lane walks the half period

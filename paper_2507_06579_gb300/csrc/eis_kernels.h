@@ -47,6 +47,16 @@ __global__ void k_walk_single(uint64_t d, const uint32_t *primes, const uint64_t
                               const uint32_t *sq_flag);
 __global__ void k_sqfree_one(uint64_t d, const uint64_t *sqtab, uint32_t nprimes, uint32_t *flag);
 
+// One membership query (k_query): what it writes to mapped host memory.
+struct QueryOut {
+    int32_t result;   // 1 + log eps_d, or -1 (error); 0: not written
+    uint32_t square;  // 1: an odd prime square divides d
+    uint32_t baby, giant;
+};
+constexpr int kQueryThreads = 256;
+__global__ void k_query(uint64_t d, const uint64_t *sqtab, uint32_t nprimes, volatile QueryOut *out,
+                        int N, int log2n, uint32_t max_rounds);
+
 __global__ void k_walk_record(const Seg *segs, uint32_t nseg, const uint32_t *surv,
                               const uint32_t *n_surv_ptr, uint32_t q_lo, uint32_t q_hi,
                               uint32_t *next_ptr, uint32_t *flags, uint8_t *glog,
