@@ -108,8 +108,11 @@ extern "C" {
                          /* (the single-query kernel)                              */
 
 /* Giant-step compositions (EIS_OPT_GIANT_COMPOSE). */
-#define EIS_COMPOSE_TEXTBOOK 0 /* product of forms, then rho until reduced      */
-                               /* (default: measured slightly faster below 2^44)*/
+#define EIS_COMPOSE_TEXTBOOK 0 /* the default: product of forms, then rho until */
+                               /* reduced (the warp-per-d kernel); the lane     */
+                               /* search and single queries reduce the product  */
+                               /* while they form it (32-bit, nearest-integer   */
+                               /* Euclid): the same ideals, sooner              */
 #define EIS_COMPOSE_NUCOMP 1   /* NUCOMP / NUDUPL / NUCOMPchoose (Algorithms    */
                                /* 2-4): near-reduced output, ~1 rho step after  */
 

@@ -260,11 +260,11 @@ static void giant_params(uint64_t d, int64_t forced, int &nbaby, int &log2n) {
 
 // Baby-step count of a single query (k_query): 256 lanes of giant steps of
 // 1.5 N steps each should reach past most periods (about 0.13 sqrt(d) steps)
-// in one round.  Mean call in us for N = 256 / 512 / 1024: 74 / 76 / 85 near
-// 10^12, 86 / 85 / 95 near 4e12, 109 / 101 / 112 near 2^44 (p99 there 241 /
-// 158 / 143).
+// in one round.  Mean call in us for N = 256 / 512 / 1024: 40 / 45 / 58 near
+// 10^11, 44 / 49 / 61 near 10^12, 49 / 53 / 66 near 4e12, 63 / 63 / 78 near 2^44
+// (p99 there 142 / 111 / 98).
 static void query_params(uint64_t d, int64_t forced, int &nbaby, int &log2n) {
-    if (forced <= 0) forced = d < 4000000000000ull ? 512 : 1024;
+    if (forced <= 0) forced = d < 2000000000000ull ? 256 : 512;
     giant_params(d, forced, nbaby, log2n);
 }
 

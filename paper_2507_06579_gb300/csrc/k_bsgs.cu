@@ -25,6 +25,7 @@
 #include "eis_bsgs.cuh"
 #include "eis_common.cuh"
 #include "eis_kernels.h"
+#include "eis_nuc.cuh"
 
 namespace eis {
 
@@ -451,11 +452,9 @@ __device__ __forceinline__ void bsgs_body(
         }
         if (fresh) {
             d = (int64_t)cand_to_d(segs, nseg, cand);
-            if (kCompose == 1) {
-                L = (int32_t)isqrt44((uint64_t)s);
-                wmu = (int32_t)lean_cG(Ideal{G.a, G.b, G.g}, d);
-            }
-            wY = (int32_t)lean_cG(Ideal{Y.a, Y.b, Y.g}, d);
+            L = (int32_t)isqrt44((uint64_t)s);
+            wmu = nuc_w(G.a, G.b, d);
+            wY = nuc_w(Y.a, Y.b, d);
             C = __uint2float_rn((uint32_t)(kFast ? 2 * s + 1 : 2 * s));
             Cw = C;
             T = __fmul_rn(tt.tau[tune_row(tt, (uint64_t)d)], __uint2float_rn((uint32_t)s));
@@ -466,26 +465,47 @@ __device__ __forceinline__ void bsgs_body(
         }
         if (!__any_sync(kFull, active)) break;
         // ---- giant step for the lanes whose last walk has ended:
-        // mu <- reduce(mu * Y), with Q_{-1} of the result, and a new walk
+        // mu <- reduce(mu * Y), with Q_{-1} of the result, and a new walk.
+        // (nuc_mul, about 400 instructions of fp32 and 32-bit integers, against
+        // 1,100 with 64-bit residues and six rho steps for the textbook product:
+        // 280 -> 188 ms for the search of the whole 10^9 window below 10^11 at
+        // N = 2048, m = 40, 17.4 -> 13.1 ms for the d that k_cubic leaves.)
         if (active && compose_now) {
-            Ideal nx{1, 1, 0};
-            int64_t Qm = 2;
-            const bool ok = bsgs_giant(kCompose, Ideal{mu.a, mu.b, mu.g}, wmu, Ideal{Y.a, Y.b, Y.g}, wY, d,
-                                       s, L, nx, Qm) &&
-                            ++cycles <= max_cycles;
-            if (!ok) {
+            NucIdeal nx{1, 1, 0, 0};
+            int st;
+            if (kCompose == 0) {
+                st = nuc_mul(NucIdeal{mu.a, mu.b, mu.g, wmu}, NucIdeal{Y.a, Y.b, Y.g, wY}, s, L, nx);
+            } else {
+                Ideal o{1, 1, 0};
+                int64_t Qm = 2;
+                st = lean_nucomp(Ideal{mu.a, mu.b, mu.g}, wmu, Ideal{Y.a, Y.b, Y.g}, wY, d, s, L, o, Qm)
+                         ? kNucOk
+                         : kNucFail;
+                nx = NucIdeal{(int32_t)o.a, (int32_t)o.b, o.g, (int32_t)(-Qm / 2)};
+            }
+            if (++cycles > max_cycles) st = kNucFail;
+            if (st == kNucFail) {
                 fallback(fb_list, fb_count, fb_cap, cand, status);
                 my_cycles += cycles;
                 active = false;
+            } else if (st == kNucRetry) {
+                // the norms share a factor: one step on, next iteration again
+                const NucIdeal m1 = nuc_step(NucIdeal{mu.a, mu.b, mu.g, wmu}, s);
+                mu = SIdeal{m1.a, m1.b, m1.g};
+                wmu = m1.w;
             } else {
-                if (first) {  // the first landing, reduce(a_jl * a_j'), is the stride
+                if (first) {
+                    // the first landing, reduce(a_jl * a_j'), is the stride (a
+                    // few steps on, at a norm without small factors)
                     first = false;
-                    Y = SIdeal{(int32_t)nx.a, (int32_t)nx.b, nx.g};
-                    wY = (int32_t)(-Qm / 2);  // (b^2 - d)/(4a) = -Q_{-1}/2
+                    const NucIdeal y1 = kCompose == 0 ? nuc_coprime(nx, s) : nx;
+                    Y = SIdeal{y1.a, y1.b, y1.g};
+                    wY = y1.w;
                 }
+                Cw = C;  // (parked while the lane waited)
                 w.num = bsgs_num(nx.b, s, kFast);
                 w.Q = __uint2float_rn((uint32_t)(2 * nx.a));
-                w.Qp = __uint2float_rn((uint32_t)Qm);
+                w.Qp = __uint2float_rn((uint32_t)(-2 * nx.w));
                 w.x = (int)((nx.b >> 1) & 1);
                 w.acc = 0;
                 gc = nx.g;
@@ -498,6 +518,7 @@ __device__ __forceinline__ void bsgs_body(
         // and one step beyond (a lane stops at x + 1); a walk that needs more
         // goes on next iteration while the other lanes compose
         bool walking = active && !compose_now;
+        const bool went = walking;
         if (!walking) lean_park_idle(w, Cw);  // idle lanes step NaN states
         uint32_t stepped = 0;
         for (uint32_t grp = 0; grp < groups && __any_sync(kFull, walking); ++grp) {
@@ -528,7 +549,7 @@ __device__ __forceinline__ void bsgs_body(
         // ---- look x up for the lanes that reached x + 1: direct key
         // (Q_x, P_x) and mirror key (Q_x, P_{x+1}); the lane stands at x + 1,
         // so Q_x = w.Qp and g_x = gc - 1 - x_{x+1}
-        const bool at_end = active && compose_now;
+        const bool at_end = went && active && compose_now;
         const uint32_t kq = __float_as_uint(w.Qp), kd = __float_as_uint(numx),
                        km = __float_as_uint(w.num);
         const bool maybe = at_end && (fp_maybe(fp_mine, kq, kd) || fp_maybe(fp_mine, kq, km));

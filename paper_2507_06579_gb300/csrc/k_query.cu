@@ -6,25 +6,28 @@
 //  * the baby walk of N steps (warp 0; about 45 clocks a step, the chain
 //    rcp -> quotient -> remainder -> Q') stores each state with one shared
 //    store; the 8 warps insert the states afterwards, 2N / 256 rounds;
-//  * 256 lanes of giant steps let N be a half of what 32 lanes want;
+//  * 256 lanes of giant steps let N be a quarter of what 32 lanes want;
 //  * lane t = 32 w + l holds mu = S^(t+1), S = reduce(a_N a_{N/2}): S^(l+1) by
 //    a scan over the lanes (5 products deep), H = S^32, H^w by another (3),
 //    and one product.  Later rounds multiply by H^8 = S^256.
-// All products are the lean product of eis_bsgs.cuh in one out-of-line copy
-// (the kernel runs once, so its instructions come from L2).
+// All products are nuc_mul (eis_nuc.cuh) in one out-of-line copy (the kernel
+// runs once, so its instructions come from L2).
 //
 // Coverage.  The table holds the window [R - delta_N, R + delta_N] whole
 // (every state, and its mirror).  S is shorter than the window by
 // delta_N - delta_{N/2}, at least N/4 pairs of steps of log 2 or more each;
 // two neighbouring powers differ by S up to the offsets of the (at most 9)
-// products they do not share, each below log 2 sqrt d.
+// products they do not share, each below log 2 sqrt d, and their few steps to
+// a norm without small factors.
 //
-// Measured, a call with its launch: 75 us against 171 us for d below 10^12,
-// 102 against 292 below 2^44 (one warp, table and giant steps alike).
+// Measured, a call with its launch: 43 us against 161 us for d below 10^12, 63
+// against 290 below 2^44 (one warp, table and giant steps alike); 75 and 102
+// with the textbook product, whose 1100 serial instructions are 5 us.
 #include "eis_common.cuh"
 #include "eis_bsgs.cuh"
 #include "eis_infra.cuh"
 #include "eis_kernels.h"
+#include "eis_nuc.cuh"
 
 namespace eis {
 
@@ -32,18 +35,29 @@ namespace {
 
 constexpr int kQWarps = kQueryThreads / 32;
 
-// Ideals as (a, b, class, w = (b^2 - d)/(4a)): reduce(X * Y); a = 0 when the
-// reduction ran away.
-__device__ __noinline__ int4 query_mul(int4 X, int4 Y, int64_t d, int64_t s) {
-    Ideal out{1, 1, 0};
-    int64_t Qm = 2;
-    const bool ok = lean_mul(Ideal{X.x, X.y, X.z}, Ideal{Y.x, Y.y, Y.z}, Y.w, d, s, out, Qm);
-    return ok ? make_int4((int)out.a, (int)out.b, out.g, (int)(-Qm / 2)) : make_int4(0, 0, 0, 0);
-}
-
-// X * Y where neither has failed.
-__device__ __forceinline__ int4 mul_ok(int4 X, int4 Y, int64_t d, int64_t s) {
-    return (X.x && Y.x) ? query_mul(X, Y, d, s) : make_int4(0, 0, 0, 0);
+// Ideals as (a, b, class, w = (b^2 - d)/(4a)): reduce(X * Y), moved on to a
+// norm without small factors; a = 0 when a factor has failed or a reduction
+// runs away.  Where the norms share a factor X steps on and tries again, and
+// after kQTries the textbook product takes the pair as it is.
+constexpr int kQTries = 6;
+__device__ __noinline__ int4 query_mul(int4 X, int4 Y, int64_t d, int32_t s, int32_t L) {
+    if (!X.x || !Y.x) return make_int4(0, 0, 0, 0);
+    NucIdeal x{X.x, X.y, X.z, X.w}, out{1, 1, 0, 0};
+    const NucIdeal y{Y.x, Y.y, Y.z, Y.w};
+    int st = kNucRetry;
+    for (int t = 0; t < kQTries && st != kNucOk; ++t) {
+        if (t) x = nuc_step(x, s);
+        st = nuc_mul(x, y, s, L, out);
+    }
+    if (st != kNucOk) {
+        Ideal o{1, 1, 0};
+        int64_t Qm = 2;
+        if (!lean_mul(Ideal{X.x, X.y, X.z}, Ideal{Y.x, Y.y, Y.z}, Y.w, d, s, o, Qm))
+            return make_int4(0, 0, 0, 0);
+        out = NucIdeal{(int32_t)o.a, (int32_t)o.b, o.g, (int32_t)(-Qm / 2)};
+    }
+    out = nuc_coprime(out, s);
+    return make_int4(out.a, out.b, out.g, out.w);
 }
 
 __device__ __forceinline__ int4 shfl4(int4 v, int src) {
@@ -137,7 +151,7 @@ __global__ void __launch_bounds__(kQueryThreads) k_query(uint64_t d, const uint6
         }
         return;
     }
-    const int64_t s = (int64_t)isqrt44(d), dd = (int64_t)d;
+    const int32_t s = (int32_t)isqrt44(d), L = (int32_t)isqrt44((uint64_t)s);
     // ---- the table: O_K again as (2, P_1), each state and its mirror
     bool ok = true;
     for (int j = 1 + tid; j <= N; j += kQueryThreads) {
@@ -154,14 +168,14 @@ __global__ void __launch_bounds__(kQueryThreads) k_query(uint64_t d, const uint6
     // ---- S, then S^(l+1) on lane l (every warp alike)
     auto state = [&](int j) {
         const float4 x = st[j];
-        return make_int4((int)x.x / 2, (int)((int64_t)x.y - s), (int)((uint32_t)__float_as_int(x.z) % 3u),
+        return make_int4((int)x.x / 2, (int)x.y - s, (int)((uint32_t)__float_as_int(x.z) % 3u),
                          -(int)st[j - 1].x / 2);
     };
-    int4 mu = query_mul(state(N), state(N / 2), dd, s);
+    int4 mu = query_mul(state(N), state(N / 2), (int64_t)d, s, L);
 #pragma unroll 1
     for (int k = 1; k < 32; k <<= 1) {
         const int4 o = shfl4(mu, lane >= k ? lane - k : lane);
-        if (lane >= k) mu = mul_ok(mu, o, dd, s);
+        if (lane >= k) mu = query_mul(mu, o, (int64_t)d, s, L);
     }
     auto found = [&](uint64_t e) {  // log eps_d from the table's entry at mu
         const int Sj = (int)(e & 3);
@@ -184,11 +198,11 @@ __global__ void __launch_bounds__(kQueryThreads) k_query(uint64_t d, const uint6
 #pragma unroll 1
     for (int k = 1; k < kQWarps; k <<= 1) {
         const int4 o = shfl4(h, lane >= k ? lane - k : lane);
-        if (lane >= k && lane < kQWarps) h = mul_ok(h, o, dd, s);
+        if (lane >= k && lane < kQWarps) h = query_mul(h, o, (int64_t)d, s, L);
     }
     const int4 stride = shfl4(h, kQWarps - 1);
     const int4 hw = shfl4(h, warp > 0 ? warp - 1 : 0);
-    if (warp > 0) mu = mul_ok(mu, hw, dd, s);
+    if (warp > 0) mu = query_mul(mu, hw, (int64_t)d, s, L);
     for (uint32_t r = 0; r < max_rounds; ++r) {
         // the first hit of the round; -1: a product failed.  (Two words in turn:
         // a round that goes on leaves its word as it was.)
@@ -207,7 +221,7 @@ __global__ void __launch_bounds__(kQueryThreads) k_query(uint64_t d, const uint6
             }
             return;
         }
-        mu = mul_ok(mu, stride, dd, s);
+        mu = query_mul(mu, stride, (int64_t)d, s, L);
     }
     if (tid == 0) out->result = -1;  // no hit within max_rounds
 }

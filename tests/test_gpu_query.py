@@ -27,7 +27,7 @@ def _ask(ctx, d):
 
 @pytest.mark.parametrize("stride", [0, 256, 4096])   # N: automatic, the least, the largest
 @pytest.mark.parametrize("lo,n", [(5, 600), (10**5, 300), (10**7, 300), (10**9, 300), (10**11, 200),
-                                  (10**12, 150), (4 * 10**12 - 400, 100),          # N 512 | 1024
+                                  (10**12, 150), (2 * 10**12 - 400, 100),          # N 256 | 512
                                   (4390000000000 - 400, 100), (E.EIS_D_LIMIT - 800, 100)])
 def test_queries_equal_the_range(ctx, lo, n, stride):
     """Every candidate of a window, square factors included."""
