@@ -11,13 +11,13 @@
 //                 nbaby.  The lane then takes the region that belongs to that
 //                 record's slot for its next d.
 //  k_bsgs_t       one d per lane, lanes refilled from the records (the warp
-//                 loads a fresh lane's table coalesced and indexes it as
-//                 fingerprints in that lane's shared memory): each cycle
-//                 composes mu <- reduce(mu * G), walks baby steps to the
-//                 first marked state x and one step beyond, and looks x up
-//                 under its direct and mirror keys (shared-memory probes; a
-//                 fingerprint match is settled by a warp-wide exact scan of
-//                 the entries); the next cycle composes from state x + 1.
+//                 loads a fresh lane's table coalesced and sets its Q's bits in
+//                 that lane's filter in shared memory): each cycle composes
+//                 mu <- reduce(mu * G), walks baby steps to the first marked
+//                 state x and one step beyond, and looks x up under its direct
+//                 and mirror keys (one probe of the filter; a match is settled
+//                 by a warp-wide exact scan of the entries); the next cycle
+//                 composes from state x + 1.
 //                 A d the search cannot finish (reduction or walk past its
 //                 limits) goes to a fallback list that the plain persistent
 //                 walk finishes.
@@ -267,48 +267,25 @@ __device__ __forceinline__ void fallback(uint32_t *fb_list, uint32_t *fb_count, 
         atomicOr(status, kErrGiant);
 }
 
-// Per-lane fingerprint index of a d's table in shared memory: 256 slots of
-// one byte, 0 = empty, else an 8-bit fingerprint (1..255) of the key stored at
-// the slot its probe sequence reached.  A key whose probe meets no slot with
-// its fingerprint before an empty one is not in the table; a fingerprint
-// match is settled by an exact scan of the entries.
-constexpr int kFpWords = kBsgsSlots / 4;
+// Per-lane filter of a d's table in shared memory: 32 words, in which every
+// entry sets two bits of one word, all three chosen by a hash of its Q (the
+// direct and the mirror key of a state share it).  A Q whose bits are not both
+// set is not in the table; a match is settled by an exact scan of the entries
+// (40 entries: 1 look-up in 170 scans in vain).
+// An entry costs one hash and one shared atomic, all 32 lanes at once.  The
+// open-addressing index of 8-bit fingerprints it replaces cost about 40,000
+// issue slots a d (probe loops and compare-and-swap retries), two thirds of the
+// search once k_cubic has left only short periods: 18.6 -> 14.4 ms for the
+// window's 1.2e7 d at N = 768, m = 24.  128 B a lane also lets 8 blocks
+// reside instead of 6.
+constexpr int kFpWords = 32;
 
-__device__ __forceinline__ uint32_t fp_of(uint32_t q, uint32_t num) {
-    const uint32_t h = (q * 0x2545F491u) ^ (num * 0x9E3779B9u) ^ (q >> 11);
-    const uint32_t f = (h * 0x85EBCA6Bu) >> 24;
-    return f ? f : 1u;
-}
-
-// Each failed compare-and-swap means another lane's insert landed in that
-// word, so with at most kBsgsKmax entries in kBsgsSlots slots an insert takes
-// fewer than kBsgsSlots + kBsgsKmax iterations; the bound is above that.
-__device__ __forceinline__ void fp_insert(uint32_t *sl, uint32_t q, uint32_t num) {
-    uint32_t p = bsgs_slot(q, num);
-    const uint32_t f = fp_of(q, num);
-    for (int n = 0; n < 2 * kBsgsSlots; ++n) {
-        const uint32_t w = p >> 2, sh = 8 * (p & 3);
-        const uint32_t cur = sl[w];
-        if ((cur >> sh) & 0xFFu) {
-            p = (p + 1) & (kBsgsSlots - 1);  // taken: next slot
-            continue;
-        }
-        if (atomicCAS(&sl[w], cur, cur | (f << sh)) == cur) return;  // else the word changed: retry
-    }
-}
-
-// True when (q, num) may be in the table (a slot on its probe sequence holds
-// its fingerprint), false when it certainly is not.
-__device__ __forceinline__ bool fp_maybe(const uint32_t *sl, uint32_t q, uint32_t num) {
-    uint32_t p = bsgs_slot(q, num);
-    const uint32_t f = fp_of(q, num);
-    for (int n = 0; n < kBsgsSlots; ++n) {
-        const uint32_t b = (sl[p >> 2] >> (8 * (p & 3))) & 0xFFu;
-        if (b == 0) return false;
-        if (b == f) return true;
-        p = (p + 1) & (kBsgsSlots - 1);
-    }
-    return true;
+__device__ __forceinline__ void fp_bits(uint32_t q, uint32_t &word, uint32_t &mask) {
+    uint32_t h = q * 0x9E3779B1u;
+    h ^= h >> 15;
+    h *= 0x2C1B3C6Du;
+    word = h >> 27;
+    mask = (1u << ((h >> 22) & 31u)) | (1u << ((h >> 17) & 31u));
 }
 
 struct SIdeal {
@@ -349,7 +326,7 @@ __device__ __forceinline__ void bsgs_body(
     float Cw = 0.0f;
     lean_park_idle(w, Cw);
     int gc = 0;
-    bool at_x = false, compose_now = false;
+    bool compose_now = false;
     float numx = 0.0f;
     uint32_t walked = 0;
     uint32_t my_cycles = 0, my_walk = 0;
@@ -376,7 +353,7 @@ __device__ __forceinline__ void bsgs_body(
             }
         }
         // ---- the whole warp indexes each fresh lane's table: entries loaded
-        // coalesced, fingerprints inserted into that lane's slots
+        // coalesced, their bits set in that lane's filter
         unsigned pend = __ballot_sync(kFull, fresh);
         while (pend) {
             const int src = __ffs(pend) - 1;
@@ -392,11 +369,14 @@ __device__ __forceinline__ void bsgs_body(
                 v[t] = i < kk ? e[i] : make_uint4(0u, 0u, 0u, 0u);
             }
             sl[lane] = 0u;
-            sl[lane + 32] = 0u;
             __syncwarp();
 #pragma unroll
             for (int t = 0; t < kBsgsKmax / 32; ++t)
-                if (lane + 32 * t < kk) fp_insert(sl, v[t].x, v[t].y);
+                if (lane + 32 * t < kk) {
+                    uint32_t word, mask;
+                    fp_bits(v[t].x, word, mask);
+                    atomicOr(&sl[word], mask);
+                }
             // G = entry kk-1, held by lane (kk-1) % 32 in v[(kk-1) / 32]
             const uint32_t tg = (kk - 1) >> 5;
             uint32_t gx = 0, gy = 0, gz = 0;
@@ -509,37 +489,37 @@ __device__ __forceinline__ void bsgs_body(
                 w.x = (int)((nx.b >> 1) & 1);
                 w.acc = 0;
                 gc = nx.g;
-                at_x = false;
                 walked = 0;
                 compose_now = false;
             }
         }
         // ---- walk at most walk_window steps toward the first marked state x
-        // and one step beyond (a lane stops at x + 1); a walk that needs more
-        // goes on next iteration while the other lanes compose
+        // and one step beyond; a walk that needs more goes on next iteration
+        // while the other lanes compose
         bool walking = active && !compose_now;
         const bool went = walking;
         if (!walking) lean_park_idle(w, Cw);  // idle lanes step NaN states
-        uint32_t stepped = 0;
+        const uint32_t walked0 = walked;
         for (uint32_t grp = 0; grp < groups && __any_sync(kFull, walking); ++grp) {
 #pragma unroll
             for (int i = 0; i < kBsgsGroup; ++i) {
                 if (walking) {
                     lean_step<kFast>(w, Cw);
-                    gc += 1 + w.x;
+                    gc += w.x;  // (the 1 per step is added at the end)
                     ++walked;
-                    ++stepped;
-                    if (at_x) {
-                        walking = false;  // at x + 1
-                        compose_now = true;
-                    } else if (w.Q < T) {
-                        at_x = true;      // at x
-                        numx = w.num;
-                    }
+                    walking = !(w.Q < T);
                 }
             }
         }
-        my_walk += stepped;
+        my_walk += walked - walked0;
+        const bool at_x = went && !walking;
+        if (at_x) {  // x + 1
+            numx = w.num;
+            lean_step<kFast>(w, Cw);
+            gc += (int)walked + 1 + w.x;
+            ++my_walk;
+            compose_now = true;
+        }
         if (active && !compose_now && walked >= walk_cap) {
             // no marked state within walk_cap steps: the fallback walk finishes it
             fallback(fb_list, fb_count, fb_cap, cand, status);
@@ -549,12 +529,14 @@ __device__ __forceinline__ void bsgs_body(
         // ---- look x up for the lanes that reached x + 1: direct key
         // (Q_x, P_x) and mirror key (Q_x, P_{x+1}); the lane stands at x + 1,
         // so Q_x = w.Qp and g_x = gc - 1 - x_{x+1}
-        const bool at_end = went && active && compose_now;
+        const bool at_end = at_x && active;
         const uint32_t kq = __float_as_uint(w.Qp), kd = __float_as_uint(numx),
                        km = __float_as_uint(w.num);
-        const bool maybe = at_end && (fp_maybe(fp_mine, kq, kd) || fp_maybe(fp_mine, kq, km));
+        uint32_t fword, fmask;
+        fp_bits(kq, fword, fmask);
+        const bool maybe = at_end && (fp_mine[fword] & fmask) == fmask;
         int g = -1;
-        // exact scan of the tables of the lanes with a fingerprint match, by
+        // exact scan of the tables of the lanes with a match, by
         // the whole warp
         unsigned scan = __ballot_sync(kFull, maybe);
         while (scan) {
@@ -620,7 +602,7 @@ __global__ void __launch_bounds__(128) k_bsgs_t(
     unsigned long long *__restrict__ acc, int *__restrict__ status, uint32_t *__restrict__ fb_list,
     uint32_t *__restrict__ fb_count, uint32_t fb_cap, const __grid_constant__ TuneTab tt,
     uint32_t max_cycles, uint32_t walk_cap, uint32_t walk_window) {
-    __shared__ uint32_t fp_all[128 * kFpWords];  // 32 KB: 256 fingerprint slots per lane
+    __shared__ uint32_t fp_all[128 * kFpWords];
     bsgs_body<kFast, kCompose>(segs, nseg, recs, nrec, rec_cap, next_ptr, pool, flags, glog, acc,
                                status, fb_list, fb_count, fb_cap, tt, max_cycles, walk_cap,
                                walk_window, fp_all);
