@@ -90,11 +90,39 @@ EIS_HD float cubic_rcp(float x) {
 #endif
 }
 
+// sqrt to a relative error below 2^-21.
 EIS_HD float cubic_sqrt(float x) {
 #ifdef __CUDA_ARCH__
-    return __fsqrt_rn(x);
+    float r;
+    asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
 #else
     return std::sqrt(x);
+#endif
+}
+
+// x y rounded to an integer next to it, |x y| < 2^22.
+EIS_HD int32_t cubic_rint(float x, float y) {
+#ifdef __CUDA_ARCH__
+    return __float_as_int(__fmaf_rn(x, y, 12582912.0f)) - 0x4B400000;
+#else
+    return (int32_t)float_bits(std::fma(x, y, 12582912.0f)) - 0x4B400000;
+#endif
+}
+
+EIS_HD int32_t cubic_ceil(float x) {
+#ifdef __CUDA_ARCH__
+    return __float2int_ru(x);
+#else
+    return (int32_t)std::ceil(x);
+#endif
+}
+
+EIS_HD int32_t cubic_floor(float x) {
+#ifdef __CUDA_ARCH__
+    return __float2int_rd(x);
+#else
+    return (int32_t)std::floor(x);
 #endif
 }
 
@@ -187,27 +215,23 @@ EIS_HD int32_t cubic_c_range(const CubicA &A, int32_t b, float plo, float phi, i
 }
 
 // The forms of one (a, b, c): Q = rho + 9a k, e = e0 - k.  Two bands of k,
-// k = k[i] + st * t for 0 <= t < n[i].
+// k = k[i] + (t << cubic_shift) for 0 <= t < n[i].
 struct CubicBands {
     int32_t P, rho, e0;
     int32_t k[2], n[2];
 };
 
-// Step of k between forms of the kind: 2, or 4 where e is fixed mod 4.
-EIS_HD int32_t cubic_step(int kind, int32_t a) { return (!kind && (a & 1)) ? 4 : 2; }
+// log2 of the step of k between forms of the kind: 1, or 2 where e is fixed
+// mod 4.
+EIS_HD int32_t cubic_shift(int kind, int32_t a) { return (!kind && (a & 1)) ? 2 : 1; }
 
 EIS_HD void cubic_one_band(const CubicA &A, float qlo, float qhi, float P, int32_t rho, int32_t kres,
-                           int32_t st, int32_t &k0, int32_t &n) {
-    n = 0;
-    k0 = 0;
-    qlo = fmaxf(qlo, -1.0f);
-    qhi = fminf(qhi, 1.0f);
-    const float m = 1.0f + 2e-6f * P;
-    const int32_t lo = (int32_t)ceilf((qlo * P - m - (float)rho) * A.r9a);
-    const int32_t hi = (int32_t)floorf((qhi * P + m - (float)rho) * A.r9a);
-    if (lo > hi || qlo * P - m > qhi * P + m) return;
-    k0 = lo + ((kres - lo) & (st - 1));
-    n = hi >= k0 ? (hi - k0) / st + 1 : 0;
+                           int32_t sh, int32_t &k0, int32_t &n) {
+    const float m = 1.0f + 2.5e-6f * P + (float)rho;
+    const int32_t lo = cubic_ceil((fmaxf(qlo, -1.0f) * P - m) * A.r9a);
+    const int32_t hi = cubic_floor((fminf(qhi, 1.0f) * P + (m - 2.0f * (float)rho)) * A.r9a);
+    k0 = lo + ((kres - lo) & ((1 << sh) - 1));
+    n = hi >= k0 ? ((hi - k0) >> sh) + 1 : 0;
 }
 
 EIS_HD void cubic_bands(const CubicA &A, int32_t b, int32_t c, CubicBands &B) {
@@ -218,39 +242,41 @@ EIS_HD void cubic_bands(const CubicA &A, int32_t b, int32_t c, CubicBands &B) {
     B.k[0] = B.k[1] = 0;
     B.rho = B.e0 = 0;
     if (P < 1) return;
-    // bc = 9a e0 + rho
-    int32_t c0;
-    const int32_t cq = cubic_floordiv(c, 9 * a, A.r9a, c0);
-    int32_t rho;
-    B.e0 = b * cq + cubic_floordiv(b * c0, 9 * a, A.r9a, rho);  // mod 2^32 is enough
+    // bc = 9a e0 + rho, rho small (e0 mod 2^32 is enough)
+    const int32_t cq = cubic_rint((float)c, A.r9a), c0 = c - 9 * a * cq;
+    const int32_t q2 = cubic_rint((float)(b * c0), A.r9a);
+    const int32_t rho = b * c0 - 9 * a * q2;
+    B.e0 = b * cq + q2;
     B.rho = rho;
-    // e == er mod st  <=>  k == e0 - er
-    const int32_t st = cubic_step(A.kind, a);
+    // e == er mod the step  <=>  k == e0 - er
+    const int32_t sh = cubic_shift(A.kind, a);
     int32_t er;
     if (A.kind)
         er = (a & b & 1) ? 0 : 1;
     else
         er = !(a & 1) ? 1 : (b & 1) ? 2 - a - b - c : 2;
     const int32_t kres = B.e0 - er;
-    // h(q) between n0 and n1
+    // h(q) between n0 and n1; u = sqrt(4b^2 - 3a n) at either end, on the side
+    // that widens n / (2b + u)
     const float fP = (float)P, rP2 = cubic_rcp(fP * fP);
     const int64_t cP2 = 4 * (int64_t)c * ((int64_t)P * P);
     const float n0 = (float)(A.K0 + cP2) * rP2, n1 = (float)(A.K1 + cP2) * rP2;
-    const float fb = 2.0f * (float)b, fa = 3.0f * (float)a;
-    const float t0 = fb * fb - fa * n0, t1 = fb * fb - fa * n1;
-    const float e0 = 1e-6f * (fb * fb + fa * fabsf(n0)), e1 = 1e-6f * (fb * fb + fa * fabsf(n1));
+    const float fb = 2.0f * (float)b, fa = 3.0f * (float)a, fb2 = fb * fb;
+    const float t0 = fb2 - fa * n0, t1 = fb2 - fa * n1;
+    const float e0 = 1e-6f * (fb2 + fa * fabsf(n0)), e1 = 1e-6f * (fb2 + fa * fabsf(n1));
     if (t0 + e0 < 0.0f) return;  // the window lies above the largest h
-    const float u0h = cubic_sqrt(t0 + e0), u0l = cubic_sqrt(fmaxf(t0 - e0, 0.0f));
-    const float u1h = cubic_sqrt(fmaxf(t1 + e1, 0.0f)), u1l = cubic_sqrt(fmaxf(t1 - e1, 0.0f));
+    const float ua = cubic_sqrt(fmaxf(n0 >= 0.0f ? t0 + e0 : t0 - e0, 0.0f));
+    const float ub = cubic_sqrt(fmaxf(n1 >= 0.0f ? t1 - e1 : t1 + e1, 0.0f));
     const float qs = fb * A.r3a;  // q*
     // below q*: q = n / (2b + u)
-    const float qa = n0 * cubic_rcp(fb + (n0 >= 0.0f ? u0h : u0l) + 1e-30f);
-    const float qb = t1 > e1 ? n1 * cubic_rcp(fb + (n1 >= 0.0f ? u1l : u1h)) : qs;
-    if (qa <= 1.000001f) cubic_one_band(A, qa, qb, fP, rho, kres, st, B.k[0], B.n[0]);
+    const float qa = n0 * cubic_rcp(fb + ua + 1e-30f);
+    const float qb = t1 > e1 ? n1 * cubic_rcp(fb + ub) : qs;
+    if (qa <= 1.00001f && qb >= -1.00001f)
+        cubic_one_band(A, qa, qb, fP, rho, kres, sh, B.k[0], B.n[0]);
     // above q*: q = (2b + u) / (3a)
-    if (qs <= 1.000001f)
-        cubic_one_band(A, (fb + u1l) * A.r3a * 0.999999f, (fb + u0h) * A.r3a * 1.000001f, fP, rho, kres,
-                       st, B.k[1], B.n[1]);
+    if (qs <= 1.00001f)
+        cubic_one_band(A, (fb + ub) * A.r3a * 0.999996f, (fb + ua) * A.r3a * 1.000004f, fP, rho, kres,
+                       sh, B.k[1], B.n[1]);
 }
 
 // The candidate (from the job's d0 on) that the form (a, b, c, e0 - k) of a

@@ -39,11 +39,12 @@ __device__ __forceinline__ int scan_owner(int32_t incl, int32_t t) {
 // lays their (b, c) out flat, 32 at a time, one per lane; the lanes' bands of
 // forms are then laid out flat again and tested 32 at a time, so that lanes
 // stay busy whether a window holds thousands of forms per (b, c) or none.
-// Bound by instruction issue (integer and conversion work per (b, c)); the
-// bitmaps stay in L2.  Measured with k_select: 1.0 ms for the 10^9 window
-// below 10^11 and 0.8 ms for one 10^6 wide, 2.6 ms near 10^12, 15.4 ms near
-// 2^44.  The window's pass went from 827 to 45 ms (walk) and from 425 to 38 ms
-// (lane search): 1.2e7 of its 1.0e8 d are left, with a third of the period.
+// Bound by instruction issue: 290 warp instructions for 32 (b, c), 83% of the
+// issue slots busy; the bitmaps stay in L2.  Measured: 0.55 ms for windows up
+// to 10^7 wide near 10^11, 1.9 ms near 10^12, about 11 ms near 2^44, and 1.0 ms
+// for the 10^9 window below 10^11, whose pass went from 827 to 45 ms (walk) and
+// from 425 to 38 ms (lane search) when the forms came in: 1.2e7 of its 1.0e8 d
+// are left, with a third of the period.
 __global__ void __launch_bounds__(256) k_cubic(const CubicJob *__restrict__ jobs, uint32_t njobs,
                                                uint32_t nunits, uint32_t *__restrict__ next_ptr,
                                                uint32_t *__restrict__ bits0,
@@ -71,7 +72,7 @@ __global__ void __launch_bounds__(256) k_cubic(const CubicJob *__restrict__ jobs
         const uint32_t nslices = cubic_slices(a);
         const int kind = (int)job.kind;
         const CubicA A = cubic_a(job, (int32_t)a);
-        const int32_t st = cubic_step(kind, A.a);
+        const int32_t sh = cubic_shift(kind, A.a);
         uint32_t *__restrict__ bits = kind ? bits1 : bits0;
         const int32_t b0 = (int32_t)(blk * kCubicBlock);
         // lanes 2i and 2i + 1 find the two ends of pair i's range of P
@@ -93,6 +94,7 @@ __global__ void __launch_bounds__(256) k_cubic(const CubicJob *__restrict__ jobs
             B.n[0] = B.n[1] = 0;
             if (item < items) cubic_bands(A, b, c, B);
             const int32_t len = B.n[0] + B.n[1];
+            if (!__any_sync(kFull, len > 0)) continue;
             const int32_t lin = warp_incl_scan(len, lane);
             const int32_t total = __shfl_sync(kFull, lin, 31);
             for (int32_t t0 = 32 * (int32_t)slice; t0 < total; t0 += 32 * (int32_t)nslices) {
@@ -104,7 +106,7 @@ __global__ void __launch_bounds__(256) k_cubic(const CubicJob *__restrict__ jobs
                 const int32_t ob = __shfl_sync(kFull, b, own), oc = __shfl_sync(kFull, c, own);
                 const int32_t oP = __shfl_sync(kFull, B.P, own), orho = __shfl_sync(kFull, B.rho, own);
                 const int32_t oe = __shfl_sync(kFull, B.e0, own);
-                const int32_t k = i < n0 ? ka + st * i : kb + st * (i - n0);
+                const int32_t k = i < n0 ? ka + (i << sh) : kb + ((i - n0) << sh);
                 if (t < total) {
                     const int64_t h = cubic_hit(kind, A.a, ob, oc, oP, orho, oe, k, job.d0, job.ncand);
                     if (h >= 0) {

@@ -22,7 +22,7 @@ int main() {
         unsigned long long triples = 0, forms = 0, pairs = 0;
         for (int a = 1; a <= (int)j.amax; ++a) {
             const CubicA A = cubic_a(j, a);
-            const int st = cubic_step(kind, a);
+            const int st = 1 << cubic_shift(kind, a);
             for (int b = 0; b < (int)j.nblk * kCubicBlock; ++b) {
                 if (!cubic_pair_ok(kind, a, b)) continue;
                 int32_t c0 = 0;
