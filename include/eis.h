@@ -75,7 +75,9 @@ extern "C" {
 #define EIS_OPT_STEP_LIMIT 4     /* per-d baby-step limit before EIS_ESTEPS   */
 #define EIS_OPT_USE_GRAPH 5      /* 1: capture plans into CUDA graphs (1)     */
 #define EIS_OPT_GIANT_THRESHOLD 6 /* baby steps after which a d is handed to  */
-                                  /* the giant-step kernel (0 = never)        */
+                                  /* the giant-step kernel (0, the default:   */
+                                  /* the library's own choice by d; never,    */
+                                  /* with EIS_OPT_STEP_LIMIT below 2^26)      */
 #define EIS_OPT_GIANT_STRIDE 7   /* giant-step stride in baby steps (0: auto) */
 #define EIS_OPT_GIANT_COMPOSE 8  /* giant-step composition: EIS_COMPOSE_*      */
 #define EIS_OPT_MEM_BUDGET 9     /* read-only: the context's device-memory    */
@@ -103,7 +105,7 @@ extern "C" {
 #define EIS_GIANT_LANE 0 /* one d per lane: the baby walk keeps the marked states  */
                          /* (Q < 1.39/mark_every * floor(sqrt d)) in a table, and   */
                          /* each giant cycle walks to a marked state and looks it  */
-                         /* up (plans of >= 2^18 candidates; smaller plans walk)   */
+                         /* up                                                     */
 #define EIS_GIANT_WARP 1 /* one d per warp: the full baby table in shared memory  */
                          /* (the single-query kernel)                              */
 

@@ -143,12 +143,19 @@ struct eis_plan {
 
 // Charge `bytes` to the context's budget; false (nothing charged) if they do
 // not fit.
+static bool pool_drop(eis_ctx *c);
+
 static bool ctx_reserve(eis_ctx *c, uint64_t bytes) {
     uint64_t cur = c->in_use.load();
     do {
-        if (bytes > c->budget || cur > c->budget - bytes) return false;
-    } while (!c->in_use.compare_exchange_weak(cur, cur + bytes));
-    return true;
+        if (bytes > c->budget) return false;
+        if (cur > c->budget - bytes) {
+            if (!pool_drop(c)) return false;  // the kept search pool gives way
+            cur = c->in_use.load();
+            continue;
+        }
+        if (c->in_use.compare_exchange_weak(cur, cur + bytes)) return true;
+    } while (true);
 }
 
 static void ctx_release(eis_ctx *c, uint64_t bytes) {
@@ -162,8 +169,11 @@ static int plan_alloc(eis_plan *p, void **ptr, size_t bytes) {
     if (!ctx_reserve(p->ctx, bytes)) return EIS_ENOMEM;
     if (cudaMalloc(ptr, bytes) != cudaSuccess) {
         cudaGetLastError();
-        ctx_release(p->ctx, bytes);
-        return EIS_ENOMEM;
+        if (!pool_drop(p->ctx) || cudaMalloc(ptr, bytes) != cudaSuccess) {
+            cudaGetLastError();
+            ctx_release(p->ctx, bytes);
+            return EIS_ENOMEM;
+        }
     }
     p->bytes += bytes;
     return EIS_OK;
@@ -206,6 +216,17 @@ static void pool_give(eis_ctx *c, unsigned char *q, uint64_t bytes) {
     c->pool_cache_bytes = bytes;
 }
 
+// Free the kept pool; false if there is none.
+static bool pool_drop(eis_ctx *c) {
+    std::lock_guard<std::mutex> lk(c->pool_mu);
+    if (!c->pool_cache) return false;
+    cudaFree(c->pool_cache);
+    ctx_release(c, c->pool_cache_bytes);
+    c->pool_cache = nullptr;
+    c->pool_cache_bytes = 0;
+    return true;
+}
+
 static uint64_t pool_cached_bytes(eis_ctx *c) {
     std::lock_guard<std::mutex> lk(c->pool_mu);
     return c->pool_cache_bytes;
@@ -230,8 +251,10 @@ static std::vector<uint32_t> odd_primes_below(uint32_t n) {
 
 // Bytes a plan needs per candidate: survivor queue (4) + two bitmaps (1/4),
 // plus the optional per-candidate log byte.
-static uint64_t max_chunk_cands(const eis_ctx *c, int with_log) {
-    const uint64_t used = c->in_use.load();
+static uint64_t max_chunk_cands(eis_ctx *c, int with_log) {
+    const uint64_t cached = pool_cached_bytes(c);  // gives way
+    const uint64_t in_use = c->in_use.load();
+    const uint64_t used = in_use > cached ? in_use - cached : 0;
     const uint64_t free_b = c->budget > used ? c->budget - used : 0;
     uint64_t m = free_b / (5 + (uint64_t)with_log + 1);
     m = std::min<uint64_t>(m, (uint64_t)1 << 31);
@@ -272,9 +295,6 @@ static constexpr int kGiantMaxLog2 = 14;  // 128 KB table per warp at most
 static constexpr uint32_t kGiantMaxRounds = 1u << 20;
 static constexpr double kTuneMargin = 0.98;  // autotuner: keep the current setting unless 2% faster
 static constexpr uint32_t kBsgsMaxCycles = 1u << 20;  // giant cycles per d before the fallback walk
-// Plans with fewer candidates than this walk every d to its centre (the
-// search's table pool is not worth allocating for them).
-static constexpr uint64_t kBsgsMinCands = (uint64_t)1 << 18;
 
 // Cubic forms are used while the step limit is at least its default, above
 // any half period below 2^44: a lower limit asks that every walk be held to
@@ -284,21 +304,47 @@ static constexpr int64_t kCubicMinStepLimit = (int64_t)1 << 26;
 // about 15 us of the whole GPU, the cost of their launches).
 static constexpr double kCubicMinGain = 4e8;
 
+// Survivors a round of the lane search holds when the settings are the
+// library's own: 4.3 GB of tables (a smaller pool than the option's default
+// for callers who never asked for the search).
+static constexpr int64_t kAutoChunk = (int64_t)1 << 21;
+
+// The lane search's own settings: baby steps N = coef d^(1/4) and about 56
+// marked states, by d in steps of 4.  Measured best N (time flat within 3% for
+// N / 1.5 .. 1.5 N): of all d 768 / 1024..1536 / 2048 / 3072..6144 near 10^10 /
+// 10^11 / 10^12 / 10^13 (coef 2.43), of the d the cubic forms leave, whose
+// periods are a third, 512 / 768..1024 / 1536 / 2048..3072 (coef 1.62).  Below
+// 5e8 (2e9 for what the forms leave) walking to the centre is as fast: 2.06
+// against 2.63 ms for 2e8 d's width at 10^9, 3.5 against 2.9 for all d.
+static void auto_rows(TuneTab &tt, bool after_forms) {
+    const double coef = after_forms ? 1.62 : 2.43;
+    double hi = after_forms ? 2e9 : 5e8;
+    const double step = after_forms ? 4.0 : 5.0;
+    tt.n = kTuneRows;
+    for (int r = 0; r < kTuneRows; ++r, hi *= step) {
+        tt.d_hi[r] = r + 1 < kTuneRows ? (uint64_t)hi : EIS_D_LIMIT;
+        const double N = coef * std::sqrt(std::sqrt(0.5 * hi));
+        tt.nbaby[r] = r == 0 ? 0u : (uint32_t)(N / 64.0 + 0.5) * 64u;
+        const double m = std::min(64.0, std::max(12.0, N / 56.0));
+        tt.tau[r] = (float)(1.39 / m);
+    }
+}
+
 // What the cubic forms save on a segment, in thread instructions (negative:
 // they cost more).  A walk takes about 0.067 sqrt(d) steps of 13.3
-// instructions (with the lane search, about 18.9 d^(1/4) steps' worth); the
-// forms decide 0.87 of the square-free d (with a log output only those in E,
-// about 0.29).  The enumeration looks at about 0.135 d^(3/4) triples for
-// kind 0 and 0.057 d^(3/4) for kind 1, whatever the window's width (counted
-// at 10^9 .. 2^44), each about 200 instructions.
+// instructions, with the lane search about 16.7 d^(1/4) steps' worth (3.1 ns a
+// d near 10^11); the forms save 0.9 of that (with a log output, where they
+// decide only d in E, 0.29).  The enumeration looks at about 0.135 d^(3/4)
+// triples for kind 0 and 0.057 d^(3/4) for kind 1, whatever the window's width
+// (counted at 10^9 .. 2^44), at about 500 instruction slots each.
 static double cubic_gain(const Seg &s, bool search, bool with_log, bool primes) {
     if (s.ncand == 0) return -1.0;
     const double d = (double)(s.d0 + 8 * (s.ncand - 1));
     double steps = 0.067 * std::sqrt(d);
-    if (search) steps = std::min(steps, 18.9 * std::sqrt(std::sqrt(d)));
+    if (search) steps = std::min(steps, 16.7 * std::sqrt(std::sqrt(d)));
     const double density = primes ? 4.0 / std::log(d) : 0.81;
-    const double walk = (double)s.ncand * density * steps * 13.3 * (with_log ? 0.29 : 0.87);
-    const double forms = 200.0 * std::pow(d, 0.75) * (with_log ? 0.135 : 0.192);
+    const double walk = (double)s.ncand * density * steps * 13.3 * (with_log ? 0.29 : 0.9);
+    const double forms = 500.0 * std::pow(d, 0.75) * (with_log ? 0.135 : 0.192);
     return 0.8 * walk - forms;
 }
 
@@ -518,9 +564,15 @@ static int plan_build(eis_ctx *c, const uint64_t *lo, const uint64_t *hi, size_t
     if (with_log) EIS_ALLOC(p->d_glog, p->total_cand);
     if (flags & EIS_PLAN_CLASSES) EIS_ALLOC(p->d_cls, 3 * nseg * sizeof(unsigned long long) + 8);
     // the settings each d of the plan takes: the context's tuning table, or
-    // one row of EIS_OPT_GIANT_THRESHOLD / EIS_OPT_MARK_EVERY
+    // one row of EIS_OPT_GIANT_THRESHOLD / EIS_OPT_MARK_EVERY, or (threshold 0,
+    // at a step limit no walk reaches) the library's own
     bool any_search = false;
-    if (!c->tune.empty()) {
+    const bool own = c->tune.empty() && c->giant_threshold == 0 && c->step_limit >= kCubicMinStepLimit;
+    if (own) {
+        auto_rows(p->tt, false);
+        for (const Seg &sg : p->segs)
+            any_search |= sg.ncand && sg.d0 + 8 * (sg.ncand - 1) >= p->tt.d_hi[0];
+    } else if (!c->tune.empty()) {
         p->tt.n = (uint32_t)c->tune.size();
         for (size_t r = 0; r < c->tune.size(); ++r) {
             p->tt.d_hi[r] = c->tune[r].d_hi;
@@ -573,23 +625,35 @@ static int plan_build(eis_ctx *c, const uint64_t *lo, const uint64_t *hi, size_t
         if (!p->cubic.empty())
             field_bytes = p->cubic.size() * sizeof(CubicJob) + nseg + 32 + (with_log ? 0 : p->nwords * 4);
     }
-    for (size_t si = 0; si < nseg; ++si)
-        left += p->cubic.empty() || !segfield[si] || with_log ? p->segs[si].ncand
-                                                               : p->segs[si].ncand * 15 / 100 + 64;
-    if (mode == EIS_MODE_PERSISTENT && any_search && p->total_cand >= kBsgsMinCands) {
+    uint64_t left_walk = 0;  // of which of segments that the forms do not decide
+    for (size_t si = 0; si < nseg; ++si) {
+        const bool plain = p->cubic.empty() || !segfield[si] || with_log;
+        left += plain ? p->segs[si].ncand : p->segs[si].ncand * 15 / 100 + 64;
+        left_walk += plain ? p->segs[si].ncand : 0;
+    }
+    if (own && left_walk < left / 2) {
+        auto_rows(p->tt, true);
+        any_search = false;
+        for (const Seg &sg : p->segs)
+            any_search |= sg.ncand && sg.d0 + 8 * (sg.ncand - 1) >= p->tt.d_hi[0];
+    }
+    if (mode == EIS_MODE_PERSISTENT && any_search && left > 0) {
         // lane-per-d search: survivors in rounds of C queue positions; the
         // pool holds one table region per resident lane plus one per d a
-        // round can hand on
-        // round, smaller when the budget left cannot hold the default round;
-        // without room for 2^16 survivors per round the plan walks instead
-        const uint64_t lanes = (uint64_t)c->sm_count * c->occ_record * 256;
+        // round can hand on; a smaller round when the budget left cannot hold
+        // the default one; without room for 2^16 survivors per round the plan
+        // walks instead
+        const uint64_t queue = (left + 31) / 32 * 32;
+        p->bsgs_grid_a = (uint32_t)std::min<uint64_t>((uint64_t)c->sm_count * c->occ_record,
+                                                      (queue + 255) / 256);
+        const uint64_t lanes = (uint64_t)p->bsgs_grid_a * 256;
         const uint64_t per_d = kBsgsRegionBytes + sizeof(DRecord) + 4;
         const uint64_t used = c->in_use.load();
         const uint64_t cached = pool_cached_bytes(c);  // reclaimable
         const uint64_t room = c->budget + cached > used + field_bytes ? c->budget + cached - used - field_bytes : 0;
         const uint64_t fit = room / per_d > lanes + 64 ? room / per_d - lanes - 64 : 0;
-        const uint64_t queue = (left + 31) / 32 * 32;
-        uint64_t C = std::min<uint64_t>((uint64_t)c->bsgs_chunk, queue);
+        uint64_t C = std::min<uint64_t>((uint64_t)(own ? std::min(c->bsgs_chunk, kAutoChunk) : c->bsgs_chunk),
+                                        queue);
         C = std::min<uint64_t>(C, fit / 32 * 32);
         if (C >= ((uint64_t)1 << 16) || C >= queue) {
             p->bsgs = 1;
@@ -597,18 +661,25 @@ static int plan_build(eis_ctx *c, const uint64_t *lo, const uint64_t *hi, size_t
             p->bsgs_window = (uint32_t)(c->bsgs_window > 0 ? c->bsgs_window : c->bsgs_walk_cap);
             p->bsgs_chunk = (uint32_t)C;
             p->bsgs_rounds = (uint32_t)((left + C - 1) / C);
-            p->bsgs_grid_a = (uint32_t)(c->sm_count * c->occ_record);
-            p->bsgs_grid_b = (uint32_t)(c->sm_count * c->occ_bsgs);
+            p->bsgs_grid_b = (uint32_t)std::min<uint64_t>((uint64_t)c->sm_count * c->occ_bsgs,
+                                                          (queue + 127) / 128);
             const uint64_t pool_need = (lanes + C) * kBsgsRegionBytes;
             uint64_t got = 0;
             p->d_pool = pool_take(c, pool_need, &got);
             if (p->d_pool) {
                 p->pool_bytes = got;  // its charge moves to this plan
                 p->bytes += got;
-            } else {
-                EIS_ALLOC(p->d_pool, pool_need);
+            } else if (plan_alloc(p, (void **)&p->d_pool, pool_need) == EIS_OK) {
                 p->pool_bytes = pool_need;
+            } else if (own) {
+                p->bsgs = 0;  // nobody asked for the search: the plan walks
+                p->d_pool = nullptr;
+            } else {
+                plan_free(p);
+                return EIS_ENOMEM;
             }
+        }
+        if (p->bsgs) {
             EIS_ALLOC(p->d_recs, C * sizeof(DRecord));
             EIS_ALLOC(p->d_fb, C * 4);
             EIS_ALLOC(p->d_bctr, 8 * sizeof(uint32_t));
@@ -1195,9 +1266,9 @@ int eis_get_tune_table(eis_ctx *c, eis_tune_row *rows, size_t cap, size_t *n_out
 // Candidate (nbaby, mark_every) pairs of the decade tuner; {0, 16} is the
 // walk alone.
 static const eis_tune_row kTuneGrid[] = {
-    {0, 0, 16},    {0, 1024, 16}, {0, 1536, 24}, {0, 2048, 24}, {0, 2048, 32},
-    {0, 2048, 40}, {0, 2304, 48}, {0, 2560, 32}, {0, 3072, 32}, {0, 3072, 40},
-    {0, 4096, 32}, {0, 4096, 48}, {0, 6144, 64}, {0, 8192, 64},
+    {0, 0, 16},    {0, 384, 12},  {0, 512, 12},  {0, 512, 16},  {0, 768, 16},
+    {0, 1024, 16}, {0, 1024, 24}, {0, 1536, 24}, {0, 2048, 24}, {0, 2048, 40},
+    {0, 3072, 32}, {0, 4096, 48}, {0, 6144, 64}, {0, 8192, 64},
 };
 
 int eis_autotune_decades(eis_ctx *c, uint64_t d_lo, uint64_t d_hi, eis_tune_row *rows_out,

@@ -67,8 +67,9 @@ def test_mixed_plan_equals_the_walk(ctx, flags, nbaby):
     """Intervals the forms decide beside others that are walked (short, empty,
     overlapping), with the lane search and without, launched twice."""
     lo, hi = W.batched_intervals(n=60, seed=21, a_range=(1e6, 1e11), len_range=(1e2, 1e5))
-    lo = [int(x) for x in lo] + [0, 5, 10**10, 10**10 + 10**6, 2 * 10**11]
-    hi = [int(x) for x in hi] + [0, 6, 10**10 + 4 * 10**6, 10**10 + 3 * 10**6 + 9, 2 * 10**11 + 2 * 10**6]
+    lo = [int(x) for x in lo] + [0, 5, 10**10, 10**10 + 10**6, 2 * 10**11, 3 * 10**9]
+    hi = [int(x) for x in hi] + [0, 6, 10**10 + 4 * 10**6, 10**10 + 3 * 10**6 + 9, 2 * 10**11 + 2 * 10**6,
+                                 3 * 10**9 + 2 * 10**7 + 1]
     ctx.set_option(E.EIS_OPT_GIANT_THRESHOLD, nbaby)
     try:
         got = []
@@ -95,7 +96,9 @@ def test_no_room_for_the_second_bitmap_walks(orc):
     """A budget that holds the plan but not the forms' bitmap: the plan is
     made all the same, and counts alike."""
     lo, n = 10**9, 1 << 20
+    walk = [(E.EIS_D_LIMIT, 0, 16)]  # no search, whose pool would take what room there is
     with E.Context(0) as c:
+        c.set_tune_table(walk)
         used0 = c.get_option(E.EIS_OPT_MEM_IN_USE)
         p = c.plan_create([lo], [lo + 8 * n])
         need = c.get_option(E.EIS_OPT_MEM_IN_USE) - used0
@@ -103,6 +106,7 @@ def test_no_room_for_the_second_bitmap_walks(orc):
         want = int(p.counts()[0])
         p.destroy()
     with E.Context(0, mem_budget_bytes=used0 + need - 64) as c:
+        c.set_tune_table(walk)
         p = c.plan_create([lo], [lo + 8 * n])
         p.launch()
         assert int(p.counts()[0]) == want
