@@ -330,6 +330,19 @@ static void auto_rows(TuneTab &tt, bool after_forms) {
     }
 }
 
+// The context's tuning table; true if any row searches.
+static bool tune_rows(const eis_ctx *c, TuneTab &tt) {
+    bool any = false;
+    tt.n = (uint32_t)c->tune.size();
+    for (size_t r = 0; r < c->tune.size(); ++r) {
+        tt.d_hi[r] = c->tune[r].d_hi;
+        tt.nbaby[r] = (uint32_t)c->tune[r].nbaby;
+        tt.tau[r] = 1.39f / (float)c->tune[r].mark_every;
+        any |= c->tune[r].nbaby > 0;
+    }
+    return any;
+}
+
 // What the cubic forms save on a segment, in thread instructions (negative:
 // they cost more).  A walk takes about 0.067 sqrt(d) steps of 13.3
 // instructions, with the lane search about 16.7 d^(1/4) steps' worth (3.1 ns a
@@ -573,13 +586,7 @@ static int plan_build(eis_ctx *c, const uint64_t *lo, const uint64_t *hi, size_t
         for (const Seg &sg : p->segs)
             any_search |= sg.ncand && sg.d0 + 8 * (sg.ncand - 1) >= p->tt.d_hi[0];
     } else if (!c->tune.empty()) {
-        p->tt.n = (uint32_t)c->tune.size();
-        for (size_t r = 0; r < c->tune.size(); ++r) {
-            p->tt.d_hi[r] = c->tune[r].d_hi;
-            p->tt.nbaby[r] = (uint32_t)c->tune[r].nbaby;
-            p->tt.tau[r] = 1.39f / (float)c->tune[r].mark_every;
-            any_search |= c->tune[r].nbaby > 0;
-        }
+        any_search = tune_rows(c, p->tt);
     } else {
         p->tt.n = 1;
         p->tt.d_hi[0] = EIS_D_LIMIT;
@@ -901,7 +908,17 @@ eis_ctx_view eis_ctx_get_view(eis_ctx *c) {
     v.giant_grid = (uint32_t)(c->sm_count * 4);
     v.giant_compose = c->giant_compose;
     v.step_limit = (uint32_t)std::min<int64_t>(c->step_limit, 0xffffffffll);
+    v.sm_count = (uint32_t)c->sm_count;
+    v.bsgs_grid = (uint32_t)(c->sm_count * c->occ_bsgs);
+    v.own_settings = c->step_limit >= kCubicMinStepLimit;
     return v;
+}
+
+void eis_ctx_search_rows(eis_ctx *c, TuneTab &tt) {
+    if (c->tune.empty())
+        auto_rows(tt, false);
+    else
+        tune_rows(c, tt);
 }
 
 void eis_giant_params(uint64_t d, int64_t forced, int &nbaby, int &log2n) {

@@ -8,6 +8,10 @@
 
 #include "eis.h"
 
+namespace eis {
+struct TuneTab;
+}
+
 struct eis_ctx_view {
     int device;
     const uint32_t *d_primes;  // odd primes < 2^22 on the device
@@ -17,7 +21,15 @@ struct eis_ctx_view {
     uint32_t giant_grid;       // one-warp blocks of k_giant that fit at once (SMs x 4)
     int giant_compose;         // EIS_COMPOSE_*
     uint32_t step_limit;
+    uint32_t sm_count;
+    uint32_t bsgs_grid;        // blocks of the lane search that fit at once
+    int own_settings;          // the step limit is at its default or above: the library
+                               // may decide d by cubic forms and search
 };
+
+// The lane search's settings for mixed batches of any d: the context's tuning
+// table, or the library's own.
+void eis_ctx_search_rows(eis_ctx *ctx, eis::TuneTab &tt);
 
 // Baby-step count and log2 table size of the giant-step search for d up to
 // `d` (forced > 0 picks the baby-step count).

@@ -73,6 +73,10 @@ struct Slot {
     int8_t *d_mem_out = nullptr, *h_mem_out = nullptr;
     unsigned char *d_mem_ctl = nullptr;  // [0] next, [8] acc[2], [24] status
     uint32_t *d_defer = nullptr;         // long walks handed to k_giant
+    // lane search (null without it)
+    DRecord *d_recs = nullptr;
+    unsigned char *d_pool = nullptr;
+    uint32_t *d_fb = nullptr, *d_bctr = nullptr;
     std::vector<Part> items;     // range segments
     std::vector<Part> members;   // membership queries
     bool busy = false;
@@ -92,6 +96,14 @@ struct eis_server {
     // finishes one long walk far sooner than a single lane (0: never)
     uint32_t defer_after = 131072;  // from eis_server_config.giant_after
     uint32_t defer_cap = 0;
+    // The lane search (eis_bsgs.cuh) takes the walks instead, in rounds of
+    // search_chunk survivors, when the server runs at its default giant_after
+    // and the slots' tables fit an eighth of the budget: 2000 requests of the
+    // serving mix at once take 48 ms against 134 (walks, and the longest handed
+    // to the warp-per-d kernel).
+    uint32_t search_chunk = 0;  // 0: walk
+    uint32_t rec_grid = 0, bsgs_grid = 0;
+    TuneTab tt{};
     std::mutex mu;
     std::condition_variable cv_work;  // dispatcher: new parts or stop
     std::condition_variable cv_done;  // waiters: a request finished
@@ -137,6 +149,13 @@ int slot_alloc(eis_server *s, Slot &sl) {
               cudaMalloc(&sl.d_defer, (size_t)s->defer_cap * 4 + 4) == cudaSuccess &&
               cudaHostAlloc(&sl.h_mem_d, S * sizeof(uint64_t), cudaHostAllocDefault) == cudaSuccess &&
               cudaHostAlloc(&sl.h_mem_out, S, cudaHostAllocDefault) == cudaSuccess;
+    if (ok && s->search_chunk) {
+        const uint64_t C = s->search_chunk;
+        ok = cudaMalloc(&sl.d_recs, C * sizeof(DRecord)) == cudaSuccess &&
+             cudaMalloc(&sl.d_pool, ((uint64_t)s->rec_grid * 256 + C) * kBsgsRegionBytes) == cudaSuccess &&
+             cudaMalloc(&sl.d_fb, C * 4) == cudaSuccess &&
+             cudaMalloc(&sl.d_bctr, 8 * sizeof(uint32_t)) == cudaSuccess;
+    }
     if (!ok) {
         cudaGetLastError();
         return EIS_ENOMEM;
@@ -148,7 +167,8 @@ void slot_free(Slot &sl) {
     if (sl.stream) cudaStreamSynchronize(sl.stream);
     void *dev[] = {sl.d_segs, sl.d_tiles, sl.d_sqfree, sl.d_flags, sl.d_tile_pop, sl.d_tile_off,
                    sl.d_surv, sl.d_ctr, sl.d_status, sl.d_counts, sl.d_steps,
-                   sl.d_mem_d, sl.d_mem_out, sl.d_mem_ctl, sl.d_defer};
+                   sl.d_mem_d, sl.d_mem_out, sl.d_mem_ctl, sl.d_defer,
+                   sl.d_recs, sl.d_pool, sl.d_fb, sl.d_bctr};
     for (void *p : dev)
         if (p) cudaFree(p);
     void *host[] = {sl.h_segs, sl.h_tiles, sl.h_counts, sl.h_status, sl.h_ctr, sl.h_mem_d,
@@ -164,6 +184,13 @@ uint64_t slot_bytes(const eis_server_config &c, uint32_t max_tiles, uint32_t def
     return words * 4 * 2 + words * 32 * 4 + (uint64_t)defer_cap * 4 +
            (uint64_t)max_tiles * (sizeof(Tile) + 8) +
            (uint64_t)c.slot_requests * (sizeof(Seg) + 16 + 9) + 320;
+}
+
+// Survivors a round of a slot's search holds, and the bytes of its tables.
+constexpr uint64_t kServeChunk = (uint64_t)1 << 18;
+
+uint64_t search_bytes(uint64_t chunk, uint32_t rec_grid) {
+    return ((uint64_t)rec_grid * 256 + chunk) * kBsgsRegionBytes + chunk * (sizeof(DRecord) + 4) + 32;
 }
 
 // Launch one batch (the slot's items) on the slot's stream.  False when any
@@ -207,12 +234,38 @@ bool launch_batch(eis_server *s, Slot &sl) {
         k_scan_tiles<<<1, 1024, 0, st>>>(sl.d_tile_pop, sl.d_tile_off, nt, sl.d_ctr);
         k_compact<<<nt, 256, 0, st>>>(sl.d_tiles, sl.d_sqfree, sl.d_tile_off, sl.d_surv, nullptr,
                                       nullptr, nullptr);
-        k_walk_persistent<<<s->grid, 256, 0, st>>>(sl.d_segs, nseg, sl.d_surv, sl.d_ctr,
-                                                   sl.d_ctr + 1, sl.d_flags, nullptr, sl.d_steps,
-                                                   sl.d_status, s->step_limit, s->defer_after,
-                                                   sl.d_defer, sl.d_ctr + 2, s->defer_cap,
-                                                   dmax < kFastDLimit ? 1 : 0);
-        if (s->defer_after) {
+        const int fast = dmax < kFastDLimit ? 1 : 0;
+        const bool search = s->search_chunk && dmax >= s->tt.d_hi[0];
+        if (search) {
+            // at most about 0.82 of the candidates are square-free; the last
+            // round takes whatever is left
+            const uint32_t C = s->search_chunk;
+            const uint32_t rounds = (uint32_t)std::max<uint64_t>(1, (cur / 100 * 82 + C - 1) / C);
+            const uint32_t ga = (uint32_t)std::min<uint64_t>(s->rec_grid, (cur + 255) / 256);
+            const uint32_t gb = (uint32_t)std::min<uint64_t>(s->bsgs_grid, (cur + 127) / 128);
+            for (uint32_t r = 0; r < rounds; ++r) {
+                const uint32_t q_lo = r * C, q_hi = r + 1 == rounds ? 0xffffffffu : q_lo + C;
+                ck(cudaMemsetAsync(sl.d_bctr, 0, 8 * sizeof(uint32_t), st));
+                k_walk_record<<<ga, 256, 0, st>>>(sl.d_segs, nseg, sl.d_surv, sl.d_ctr, q_lo, q_hi,
+                                                  sl.d_bctr, sl.d_flags, nullptr, sl.d_steps,
+                                                  sl.d_status, s->step_limit, s->tt, sl.d_recs,
+                                                  sl.d_bctr + 1, C, sl.d_pool, sl.d_steps + 3, fast);
+                ck(launch_k_bsgs(gb, st, fast, cv.giant_compose, sl.d_segs, nseg, sl.d_recs,
+                                 sl.d_bctr + 1, C, sl.d_bctr + 3, sl.d_pool, sl.d_flags, nullptr,
+                                 sl.d_steps + 1, sl.d_status, sl.d_fb, sl.d_bctr + 4, C, s->tt,
+                                 1u << 20, 1u << 14, 64));
+                k_walk_persistent<<<s->grid, 256, 0, st>>>(sl.d_segs, nseg, sl.d_fb, sl.d_bctr + 4,
+                                                           sl.d_bctr + 5, sl.d_flags, nullptr,
+                                                           sl.d_steps, sl.d_status, s->step_limit, 0u,
+                                                           nullptr, nullptr, 0u, fast);
+            }
+        } else {
+            k_walk_persistent<<<s->grid, 256, 0, st>>>(sl.d_segs, nseg, sl.d_surv, sl.d_ctr,
+                                                       sl.d_ctr + 1, sl.d_flags, nullptr, sl.d_steps,
+                                                       sl.d_status, s->step_limit, s->defer_after,
+                                                       sl.d_defer, sl.d_ctr + 2, s->defer_cap, fast);
+        }
+        if (s->defer_after && !search) {
             int nbaby, log2n;
             eis_giant_params(dmax, 0, nbaby, log2n);
             k_giant<<<s->giant_grid, 32, (size_t)8 << log2n, st>>>(
@@ -428,7 +481,8 @@ int eis_server_create(eis_ctx *ctx, const eis_server_config *cfg, eis_server **o
         c.giant_max = cfg->giant_max;
         c.fail_launches = cfg->fail_launches;
     }
-    if (c.giant_after == 0) c.giant_after = 131072;
+    const bool own_after = c.giant_after == 0;
+    if (own_after) c.giant_after = 131072;
     if (c.slots > 64 || c.slot_candidates < 64 || c.slot_candidates > ((uint64_t)1 << 30) ||
         c.slot_requests < 1)
         return EIS_EINVAL;
@@ -449,21 +503,50 @@ int eis_server_create(eis_ctx *ctx, const eis_server_config *cfg, eis_server **o
     // lower measured no better at p99).
     s->defer_cap = c.giant_max ? c.giant_max
                                : (uint32_t)std::max<uint64_t>(1024, c.slot_candidates / 8);
-    const uint64_t need = slot_bytes(c, s->max_tiles, s->defer_cap) * c.slots;
+    uint64_t need = slot_bytes(c, s->max_tiles, s->defer_cap) * c.slots;
     if (!eis_ctx_reserve(ctx, need)) {
         delete s;
         return EIS_ENOMEM;
     }
+    if (own_after && v.own_settings) {
+        int64_t budget = 0;
+        eis_get_option(ctx, EIS_OPT_MEM_BUDGET, &budget);
+        s->rec_grid = v.sm_count * 2;
+        s->bsgs_grid = v.bsgs_grid;
+        const uint64_t C = std::min<uint64_t>(kServeChunk, c.slot_candidates + 32ull * c.slot_requests);
+        const uint64_t more = search_bytes(C, s->rec_grid) * c.slots;
+        if (more <= (uint64_t)budget / 8 && eis_ctx_reserve(ctx, more)) {
+            s->search_chunk = (uint32_t)C;
+            need += more;
+            eis_ctx_search_rows(ctx, s->tt);
+        }
+    }
     s->st.reserved_bytes = need;
     s->slots.resize(c.slots);
-    for (Slot &sl : s->slots) {
-        int rc = slot_alloc(s, sl);
-        if (rc != EIS_OK) {
-            for (Slot &x : s->slots) slot_free(x);
-            eis_ctx_release(ctx, need);
-            delete s;
-            return rc;
-        }
+    auto alloc_slots = [&]() {
+        int rc = EIS_OK;
+        for (Slot &sl : s->slots)
+            if (rc == EIS_OK) rc = slot_alloc(s, sl);
+        if (rc != EIS_OK)
+            for (Slot &x : s->slots) {
+                slot_free(x);
+                x = Slot();
+            }
+        return rc;
+    };
+    int rc = alloc_slots();
+    if (rc == EIS_ENOMEM && s->search_chunk) {  // without the search's tables, then
+        const uint64_t more = search_bytes(s->search_chunk, s->rec_grid) * c.slots;
+        eis_ctx_release(ctx, more);
+        need -= more;
+        s->st.reserved_bytes = need;
+        s->search_chunk = 0;
+        rc = alloc_slots();
+    }
+    if (rc != EIS_OK) {
+        eis_ctx_release(ctx, need);
+        delete s;
+        return rc;
     }
     s->th = std::thread(dispatcher, s);
     *out = s;
