@@ -54,6 +54,12 @@ struct eis_ctx {
     // bytes stay charged to in_use): freeing and mapping tens of GB per plan
     // cost milliseconds in every eis_classify_range / eis_count_range call.
     std::mutex pool_mu;
+    // Plans' buffers come from this memory pool, which keeps up to
+    // kMempoolKeep freed bytes mapped: with cudaMalloc and cudaFree (a dozen a
+    // plan) a call over a short range spent most of its time on them.
+    cudaMemPool_t mempool = nullptr;
+    cudaStream_t aux = nullptr;      // allocations and table copies (never behind a launch)
+    unsigned char *h_res = nullptr;  // pinned: a plan's results on their way to the host
     unsigned char *pool_cache = nullptr;
     uint64_t pool_cache_bytes = 0;
     int mode = EIS_MODE_PERSISTENT;
@@ -76,6 +82,9 @@ struct eis_ctx {
     std::vector<eis_tune_row> tune;         // per-decade lane-search settings (empty: none)
     eis_stats last{};
 };
+
+static constexpr uint64_t kMempoolKeep = (uint64_t)1 << 30;
+static constexpr size_t kPinnedRes = 256 << 10;
 
 struct PlainBlock {
     uint64_t d_first, cand_first;
@@ -137,6 +146,12 @@ struct eis_plan {
     cudaEvent_t ev[5] = {nullptr, nullptr, nullptr, nullptr, nullptr};
     cudaStream_t last_stream = nullptr;
     bool launched = false;
+    // the tables [segs | tiles | cubic jobs | segfield] and the results
+    // [status | ctr | steps | counts | cls], one allocation and one copy each
+    unsigned char *d_tab = nullptr, *d_res = nullptr;
+    size_t res_bytes = 0;
+    std::vector<unsigned char> res;  // host copy of the last launch's results
+    bool fetched = false;
 };
 
 // ------------------------------------------------------------------ helpers
@@ -164,19 +179,26 @@ static void ctx_release(eis_ctx *c, uint64_t bytes) {
     }
 }
 
-static int plan_alloc(eis_plan *p, void **ptr, size_t bytes) {
+// Device memory for a plan, charged to the context: from its memory pool in
+// the order of its aux stream (plan_build waits for it before it returns),
+// or, for the search's tables, mapped on its own.
+static int plan_alloc(eis_plan *p, void **ptr, size_t bytes, bool own = false) {
     if (bytes == 0) bytes = 16;
-    if (!ctx_reserve(p->ctx, bytes)) return EIS_ENOMEM;
-    if (cudaMalloc(ptr, bytes) != cudaSuccess) {
-        cudaGetLastError();
-        if (!pool_drop(p->ctx) || cudaMalloc(ptr, bytes) != cudaSuccess) {
-            cudaGetLastError();
-            ctx_release(p->ctx, bytes);
-            return EIS_ENOMEM;
+    eis_ctx *c = p->ctx;
+    if (!ctx_reserve(c, bytes)) return EIS_ENOMEM;
+    for (int t = 0; t < 2; ++t) {
+        const cudaError_t e = own ? cudaMalloc(ptr, bytes)
+                                  : cudaMallocFromPoolAsync(ptr, bytes, c->mempool, c->aux);
+        if (e == cudaSuccess) {
+            p->bytes += bytes;
+            return EIS_OK;
         }
+        cudaGetLastError();
+        *ptr = nullptr;
+        if (!pool_drop(c)) break;
     }
-    p->bytes += bytes;
-    return EIS_OK;
+    ctx_release(c, bytes);
+    return EIS_ENOMEM;
 }
 
 // The cached search pool if it holds at least `bytes` (its charge moves to the
@@ -376,12 +398,8 @@ static int plan_enqueue(eis_plan *p, cudaStream_t s, bool capturing) {
     int launches = 0;
     record(p->ev[0], s, capturing);
     EIS_CK(cudaMemsetAsync(p->d_flags, 0, p->nwords * 4, s));
-    EIS_CK(cudaMemsetAsync(p->d_ctr, 0, 8 * sizeof(uint32_t), s));
-    EIS_CK(cudaMemsetAsync(p->d_status, 0, sizeof(int), s));
-    EIS_CK(cudaMemsetAsync(p->d_counts, 0, 2 * nseg * sizeof(unsigned long long) + 8, s));
-    EIS_CK(cudaMemsetAsync(p->d_steps, 0, 4 * sizeof(unsigned long long), s));
+    EIS_CK(cudaMemsetAsync(p->d_res, 0, p->res_bytes, s));
     if (p->d_glog) EIS_CK(cudaMemsetAsync(p->d_glog, 0, p->total_cand, s));
-    if (p->d_cls) EIS_CK(cudaMemsetAsync(p->d_cls, 0, 3 * nseg * sizeof(unsigned long long) + 8, s));
     if (ntiles > 0) {
         k_sieve<<<ntiles, 256, 0, s>>>(p->d_tiles, p->d_segs, c->d_primes, c->nprimes, p->d_sqfree,
                                        p->d_tile_pop, p->primes_only);
@@ -473,34 +491,32 @@ static int plan_enqueue(eis_plan *p, cudaStream_t s, bool capturing) {
     return EIS_OK;
 }
 
-static void plan_free(eis_plan *p) {
+// Free a plan.  idle: no kernel of the plan is running on any stream; else the
+// device is waited for, as cudaFree would.
+static void plan_free(eis_plan *p, bool idle = false) {
     if (!p) return;
+    eis_ctx *c = p->ctx;
     if (p->exec) cudaGraphExecDestroy(p->exec);
     if (p->graph) cudaGraphDestroy(p->graph);
     for (auto &e : p->ev)
         if (e) cudaEventDestroy(e);
     for (auto &e : p->bev)
         if (e) cudaEventDestroy(e);
-    if (p->d_pool && p->ctx) {
-        // the pool goes to the context's cache; wait for any kernel still
-        // using it (as cudaFree would)
-        cudaDeviceSynchronize();
-        pool_give(p->ctx, p->d_pool, p->pool_bytes);
+    if (!idle) cudaDeviceSynchronize();
+    if (p->d_pool) {
+        pool_give(c, p->d_pool, p->pool_bytes);  // kept for the next plan
         p->bytes -= std::min(p->bytes, p->pool_bytes);
-        p->d_pool = nullptr;
     }
-    void *bufs[] = {p->d_segs, p->d_tiles, p->d_sqfree, p->d_flags, p->d_tile_pop, p->d_tile_off,
-                    p->d_surv, p->d_ctr, p->d_status, p->d_counts, p->d_steps, p->d_glog,
-                    p->d_defer, p->d_cls, p->d_recs, p->d_pool, p->d_fb, p->d_bctr,
-                    p->d_cubic, p->d_field, p->d_segfield};
+    void *bufs[] = {p->d_tab, p->d_res, p->d_sqfree, p->d_flags, p->d_tile_pop, p->d_tile_off, p->d_surv,
+                    p->d_glog, p->d_defer, p->d_recs, p->d_fb, p->d_bctr, p->d_field};
     for (void *b : bufs)
-        if (b) cudaFree(b);
-    if (p->ctx) ctx_release(p->ctx, p->bytes);
+        if (b) cudaFreeAsync(b, c->aux);
+    ctx_release(c, p->bytes);
     delete p;
 }
 
 static int plan_build(eis_ctx *c, const uint64_t *lo, const uint64_t *hi, size_t n, int mode,
-                      int with_log, eis_plan **out, uint32_t flags = 0) {
+                      int with_log, eis_plan **out, uint32_t flags = 0, bool one_shot = false) {
     EisNvtxRange range("eis.plan_build");
     if (flags & ~(uint32_t)(EIS_PLAN_CLASSES | EIS_PLAN_PRIMES)) return EIS_EINVAL;
     if (flags & EIS_PLAN_CLASSES) with_log = 1;
@@ -563,19 +579,21 @@ static int plan_build(eis_ctx *c, const uint64_t *lo, const uint64_t *hi, size_t
             return rc;                                                    \
         }                                                                 \
     } while (0)
-    EIS_ALLOC(p->d_segs, nseg * sizeof(Seg));
-    EIS_ALLOC(p->d_tiles, ntiles * sizeof(Tile));
     EIS_ALLOC(p->d_sqfree, p->nwords * 4);
     EIS_ALLOC(p->d_flags, p->nwords * 4);
     EIS_ALLOC(p->d_tile_pop, ntiles * 4);
     EIS_ALLOC(p->d_tile_off, ntiles * 4);
     if (mode == EIS_MODE_PERSISTENT) EIS_ALLOC(p->d_surv, p->total_cand * 4);
-    EIS_ALLOC(p->d_ctr, 8 * sizeof(uint32_t));
-    EIS_ALLOC(p->d_status, sizeof(int));
-    EIS_ALLOC(p->d_counts, 2 * nseg * sizeof(unsigned long long) + 8);
-    EIS_ALLOC(p->d_steps, 4 * sizeof(unsigned long long));
+    const size_t nres = 16 + 8 * sizeof(uint32_t) + 4 * 8 + (2 * nseg + 1) * 8 +
+                        ((flags & EIS_PLAN_CLASSES) ? (3 * nseg + 1) * 8 : 0);
+    EIS_ALLOC(p->d_res, nres);
+    p->res_bytes = nres;
+    p->d_status = reinterpret_cast<int *>(p->d_res);
+    p->d_ctr = reinterpret_cast<uint32_t *>(p->d_res + 16);
+    p->d_steps = reinterpret_cast<unsigned long long *>(p->d_res + 48);
+    p->d_counts = p->d_steps + 4;
+    if (flags & EIS_PLAN_CLASSES) p->d_cls = p->d_counts + 2 * nseg + 1;
     if (with_log) EIS_ALLOC(p->d_glog, p->total_cand);
-    if (flags & EIS_PLAN_CLASSES) EIS_ALLOC(p->d_cls, 3 * nseg * sizeof(unsigned long long) + 8);
     // the settings each d of the plan takes: the context's tuning table, or
     // one row of EIS_OPT_GIANT_THRESHOLD / EIS_OPT_MARK_EVERY, or (threshold 0,
     // at a step limit no walk reaches) the library's own
@@ -676,7 +694,7 @@ static int plan_build(eis_ctx *c, const uint64_t *lo, const uint64_t *hi, size_t
             if (p->d_pool) {
                 p->pool_bytes = got;  // its charge moves to this plan
                 p->bytes += got;
-            } else if (plan_alloc(p, (void **)&p->d_pool, pool_need) == EIS_OK) {
+            } else if (plan_alloc(p, (void **)&p->d_pool, pool_need, true) == EIS_OK) {
                 p->pool_bytes = pool_need;
             } else if (own) {
                 p->bsgs = 0;  // nobody asked for the search: the plan walks
@@ -710,19 +728,32 @@ static int plan_build(eis_ctx *c, const uint64_t *lo, const uint64_t *hi, size_t
         }
         p->giant_grid = (uint32_t)(c->sm_count * std::max(1, occ));
     }
-    if (!p->cubic.empty()) {
-        // without room for them the plan walks every d
-        if (plan_alloc(p, (void **)&p->d_cubic, p->cubic.size() * sizeof(CubicJob)) != EIS_OK ||
-            plan_alloc(p, (void **)&p->d_segfield, nseg) != EIS_OK ||
-            (!with_log && plan_alloc(p, (void **)&p->d_field, p->nwords * 4) != EIS_OK)) {
-            p->cubic.clear();
-        } else if (cudaMemcpy(p->d_cubic, p->cubic.data(), p->cubic.size() * sizeof(CubicJob),
-                              cudaMemcpyHostToDevice) != cudaSuccess ||
-                   cudaMemcpy(p->d_segfield, segfield.data(), nseg, cudaMemcpyHostToDevice) != cudaSuccess) {
+    {
+        const size_t o_tiles = nseg * sizeof(Seg), o_cubic = o_tiles + ntiles * sizeof(Tile),
+                     o_field = o_cubic + p->cubic.size() * sizeof(CubicJob);
+        std::vector<unsigned char> h(o_field + nseg);
+        if (nseg) std::memcpy(h.data(), p->segs.data(), nseg * sizeof(Seg));
+        if (ntiles) std::memcpy(h.data() + o_tiles, p->tiles.data(), ntiles * sizeof(Tile));
+        if (!p->cubic.empty())
+            std::memcpy(h.data() + o_cubic, p->cubic.data(), p->cubic.size() * sizeof(CubicJob));
+        if (nseg) std::memcpy(h.data() + o_field, segfield.data(), nseg);
+        EIS_ALLOC(p->d_tab, h.size());
+        p->d_segs = reinterpret_cast<Seg *>(p->d_tab);
+        p->d_tiles = reinterpret_cast<Tile *>(p->d_tab + o_tiles);
+        p->d_cubic = reinterpret_cast<CubicJob *>(p->d_tab + o_cubic);
+        p->d_segfield = p->d_tab + o_field;
+        // (the stream's allocations are complete, and the copy done, after the wait)
+        if ((!h.empty() && cudaMemcpyAsync(p->d_tab, h.data(), h.size(), cudaMemcpyHostToDevice,
+                                           c->aux) != cudaSuccess) ||
+            cudaStreamSynchronize(c->aux) != cudaSuccess) {
             plan_free(p);
             return EIS_EDEVICE;
         }
     }
+    // without room for its bitmap the plan does without the forms
+    if (!p->cubic.empty() && !with_log &&
+        plan_alloc(p, (void **)&p->d_field, p->nwords * 4) != EIS_OK)
+        p->cubic.clear();
 #undef EIS_ALLOC
     for (auto &e : p->ev) {
         if (cudaEventCreate(&e) != cudaSuccess) {
@@ -736,17 +767,9 @@ static int plan_build(eis_ctx *c, const uint64_t *lo, const uint64_t *hi, size_t
             return EIS_EDEVICE;
         }
     }
-    if (nseg && cudaMemcpy(p->d_segs, p->segs.data(), nseg * sizeof(Seg), cudaMemcpyHostToDevice) != cudaSuccess) {
-        plan_free(p);
-        return EIS_EDEVICE;
-    }
-    if (ntiles && cudaMemcpy(p->d_tiles, p->tiles.data(), ntiles * sizeof(Tile), cudaMemcpyHostToDevice) != cudaSuccess) {
-        plan_free(p);
-        return EIS_EDEVICE;
-    }
     const int per_sm = c->ctas_per_sm > 0 ? c->ctas_per_sm : c->occ_persistent;
     p->walk_grid = (uint32_t)(c->sm_count * std::max(1, per_sm));
-    if (c->use_graph) {
+    if (c->use_graph && !one_shot) {
         cudaGraph_t g = nullptr;
         if (cudaStreamBeginCapture(c->stream, cudaStreamCaptureModeThreadLocal) != cudaSuccess) {
             plan_free(p);
@@ -782,27 +805,44 @@ static int plan_launch(eis_plan *p, cudaStream_t s) {
     }
     p->last_stream = s;
     p->launched = true;
+    p->fetched = false;
     return EIS_OK;
 }
 
+// Wait for the last launch and bring its results (p->res) to the host, once.
 static int plan_wait(eis_plan *p) {
     if (!p->launched) return EIS_EINVAL;
-    EIS_CK(cudaStreamSynchronize(p->last_stream));
+    if (!p->fetched) {
+        unsigned char *pinned = p->res_bytes <= kPinnedRes ? p->ctx->h_res : nullptr;
+        p->res.resize(p->res_bytes);
+        EIS_CK(cudaMemcpyAsync(pinned ? pinned : p->res.data(), p->d_res, p->res_bytes,
+                               cudaMemcpyDeviceToHost, p->last_stream));
+        EIS_CK(cudaStreamSynchronize(p->last_stream));
+        if (pinned) std::memcpy(p->res.data(), pinned, p->res_bytes);
+        p->fetched = true;
+    }
     int status = 0;
-    EIS_CK(cudaMemcpy(&status, p->d_status, sizeof(int), cudaMemcpyDeviceToHost));
+    std::memcpy(&status, p->res.data(), sizeof(int));
     if (status & (kErrSteps | kErrGiant)) return EIS_ESTEPS;
     return EIS_OK;
+}
+
+// The n words of the fetched results that the device holds at `at`.
+template <class T>
+static std::vector<T> plan_result(const eis_plan *p, const T *at, size_t n) {
+    std::vector<T> v(n);
+    if (n)
+        std::memcpy(v.data(), p->res.data() + (reinterpret_cast<const unsigned char *>(at) - p->d_res),
+                    n * sizeof(T));
+    return v;
 }
 
 static int plan_fill_stats(eis_plan *p, eis_stats *st) {
     int rc = plan_wait(p);
     if (rc != EIS_OK) return rc;
     std::memset(st, 0, sizeof(*st));
-    unsigned long long steps[4] = {0, 0, 0, 0};
-    EIS_CK(cudaMemcpy(steps, p->d_steps, sizeof(steps), cudaMemcpyDeviceToHost));
-    std::vector<unsigned long long> cnt(2 * p->segs.size() + 1);
-    EIS_CK(cudaMemcpy(cnt.data(), p->d_counts, cnt.size() * sizeof(unsigned long long),
-                      cudaMemcpyDeviceToHost));
+    const std::vector<unsigned long long> steps = plan_result(p, p->d_steps, 4);
+    const std::vector<unsigned long long> cnt = plan_result(p, p->d_counts, 2 * p->segs.size());
     for (size_t i = 0; i < p->segs.size(); ++i) {
         st->candidates += p->segs[i].ncand;
         st->in_E += cnt[2 * i];
@@ -810,8 +850,7 @@ static int plan_fill_stats(eis_plan *p, eis_stats *st) {
     }
     st->baby_steps = steps[0] + steps[1];
     st->giant_steps = steps[2];
-    uint32_t ctr[4] = {0, 0, 0, 0};
-    EIS_CK(cudaMemcpy(ctr, p->d_ctr, sizeof(ctr), cudaMemcpyDeviceToHost));
+    const std::vector<uint32_t> ctr = plan_result(p, p->d_ctr, 4);
     st->deferred = p->d_defer ? std::min(ctr[2], p->defer_cap) : 0;
     if (p->bsgs) {
         // steps[0]: baby steps of the recording and fallback walks, [1]: steps
@@ -845,9 +884,7 @@ static int plan_fill_stats(eis_plan *p, eis_stats *st) {
 static int plan_counts_user(eis_plan *p, uint64_t *counts_out) {
     int rc = plan_wait(p);
     if (rc != EIS_OK) return rc;
-    std::vector<unsigned long long> cnt(2 * p->segs.size() + 1);
-    EIS_CK(cudaMemcpy(cnt.data(), p->d_counts, cnt.size() * sizeof(unsigned long long),
-                      cudaMemcpyDeviceToHost));
+    const std::vector<unsigned long long> cnt = plan_result(p, p->d_counts, 2 * p->segs.size());
     for (size_t i = 0; i < p->segs.size(); ++i) counts_out[p->user_of[i]] = cnt[2 * i];
     return EIS_OK;
 }
@@ -869,13 +906,13 @@ static int run_chunks(eis_ctx *c, uint64_t lo, uint64_t hi, int with_log, cudaSt
         const uint64_t a = lo + 8 * off;
         const uint64_t b = std::min(hi, lo + 8 * (off + M));
         eis_plan *p = nullptr;
-        int rc = plan_build(c, &a, &b, 1, c->mode, with_log, &p);
+        int rc = plan_build(c, &a, &b, 1, c->mode, with_log, &p, 0, true);
         if (rc != EIS_OK) return rc;
         rc = plan_launch(p, s);
         eis_stats st{};
         if (rc == EIS_OK) rc = plan_fill_stats(p, &st);
         if (rc == EIS_OK) rc = on_chunk(p, off);
-        plan_free(p);
+        plan_free(p, rc == EIS_OK);  // (every step waits for its stream)
         if (rc != EIS_OK) return rc;
         acc->candidates += st.candidates;
         acc->in_D += st.in_D;
@@ -973,9 +1010,23 @@ int eis_create(eis_ctx **out, int device, uint64_t mem_budget_bytes) {
         return EIS_EDEVICE;
     }
     c->budget = mem_budget_bytes ? mem_budget_bytes : (uint64_t)free_b / 4 * 3;
-    if (cudaStreamCreateWithFlags(&c->stream, cudaStreamNonBlocking) != cudaSuccess) {
+    if (cudaStreamCreateWithFlags(&c->stream, cudaStreamNonBlocking) != cudaSuccess ||
+        cudaStreamCreateWithFlags(&c->aux, cudaStreamNonBlocking) != cudaSuccess) {
         delete c;
         return EIS_EDEVICE;
+    }
+    {
+        cudaMemPoolProps mp = {};
+        mp.allocType = cudaMemAllocationTypePinned;
+        mp.location.type = cudaMemLocationTypeDevice;
+        mp.location.id = device;
+        uint64_t keep = std::min<uint64_t>(kMempoolKeep, c->budget);
+        if (cudaMemPoolCreate(&c->mempool, &mp) != cudaSuccess ||
+            cudaMemPoolSetAttribute(c->mempool, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess ||
+            cudaHostAlloc(&c->h_res, kPinnedRes, cudaHostAllocDefault) != cudaSuccess) {
+            eis_destroy(c);
+            return EIS_EDEVICE;
+        }
     }
     std::vector<uint32_t> pr = odd_primes_below(1u << 22);
     c->nprimes = (uint32_t)pr.size();
@@ -1056,9 +1107,12 @@ int eis_destroy(eis_ctx *c) {
     if (c->d_single) cudaFree(c->d_single);
     if (c->d_query) cudaFree(c->d_query);
     if (c->h_query) cudaFreeHost(c->h_query);
+    if (c->h_res) cudaFreeHost(c->h_res);
+    if (c->mempool) cudaMemPoolDestroy(c->mempool);
     if (c->d_sqtab) cudaFree(c->d_sqtab);
     if (c->pool_cache) cudaFree(c->pool_cache);
     if (c->stream) cudaStreamDestroy(c->stream);
+    if (c->aux) cudaStreamDestroy(c->aux);
     delete c;
     return EIS_OK;
 }
@@ -1165,9 +1219,7 @@ int eis_plan_class_counts(eis_plan *p, uint64_t *out) {
     if (!p->d_cls) return EIS_EINVAL;
     int rc = plan_wait(p);
     if (rc != EIS_OK) return rc;
-    std::vector<unsigned long long> cnt(3 * p->segs.size() + 1);
-    EIS_CK(cudaMemcpy(cnt.data(), p->d_cls, cnt.size() * sizeof(unsigned long long),
-                      cudaMemcpyDeviceToHost));
+    const std::vector<unsigned long long> cnt = plan_result(p, p->d_cls, 3 * p->segs.size());
     for (size_t i = 0; i < p->segs.size(); ++i)
         for (int g = 0; g < 3; ++g) out[3 * p->user_of[i] + g] = cnt[3 * i + g];
     return EIS_OK;
@@ -1189,12 +1241,12 @@ int eis_class_counts(eis_ctx *c, uint64_t lo, uint64_t hi, int primes_only, uint
         eis_plan *p = nullptr;
         int rc = plan_build(c, &a, &b, 1, c->mode == EIS_MODE_PLAIN ? EIS_MODE_PLAIN
                                                                      : EIS_MODE_PERSISTENT,
-                            1, &p, flags);
+                            1, &p, flags, true);
         if (rc != EIS_OK) return rc;
         rc = plan_launch(p, c->stream);
         uint64_t part[3] = {0, 0, 0};
         if (rc == EIS_OK) rc = eis_plan_class_counts(p, part);
-        plan_free(p);
+        plan_free(p, rc == EIS_OK);
         if (rc != EIS_OK) return rc;
         for (int g = 0; g < 3; ++g) acc[g] += part[g];
     }
@@ -1216,9 +1268,7 @@ int eis_plan_counts_D(eis_plan *p, uint64_t *counts_D_out) {
     if (!p || (!counts_D_out && p->n)) return EIS_EINVAL;
     int rc = plan_wait(p);
     if (rc != EIS_OK) return rc;
-    std::vector<unsigned long long> cnt(2 * p->segs.size() + 1);
-    EIS_CK(cudaMemcpy(cnt.data(), p->d_counts, cnt.size() * sizeof(unsigned long long),
-                      cudaMemcpyDeviceToHost));
+    const std::vector<unsigned long long> cnt = plan_result(p, p->d_counts, 2 * p->segs.size());
     for (size_t i = 0; i < p->segs.size(); ++i) counts_D_out[p->user_of[i]] = cnt[2 * i + 1];
     return EIS_OK;
 }
@@ -1520,7 +1570,7 @@ int eis_classify_range_u8(eis_ctx *c, uint64_t lo, uint64_t hi, uint8_t *codes_o
         if (n == 0) return EIS_OK;
         uint8_t *tmp = out_on_device ? codes_out + off : nullptr;
         if (!tmp) {
-            if (cudaMalloc(&tmp, n) != cudaSuccess) {
+            if (cudaMallocFromPoolAsync(reinterpret_cast<void **>(&tmp), n, c->mempool, s) != cudaSuccess) {
                 cudaGetLastError();
                 return EIS_ENOMEM;
             }
@@ -1531,7 +1581,7 @@ int eis_classify_range_u8(eis_ctx *c, uint64_t lo, uint64_t hi, uint8_t *codes_o
         if (e == cudaSuccess && !out_on_device)
             e = cudaMemcpyAsync(codes_out + off, tmp, n, cudaMemcpyDeviceToHost, s);
         if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-        if (!out_on_device) cudaFree(tmp);
+        if (!out_on_device) cudaFreeAsync(tmp, c->aux);  // (the stream has been waited for)
         (void)kind;
         return e == cudaSuccess ? EIS_OK : EIS_EDEVICE;
     });
@@ -1699,14 +1749,14 @@ int eis_count_batch(eis_ctx *c, const uint64_t *lo, const uint64_t *hi, size_t n
         }
         if (gidx.empty()) continue;
         eis_plan *p = nullptr;
-        int rc = plan_build(c, glo.data(), ghi.data(), glo.size(), c->mode, 0, &p);
+        int rc = plan_build(c, glo.data(), ghi.data(), glo.size(), c->mode, 0, &p, 0, true);
         if (rc != EIS_OK) return rc;
         rc = plan_launch(p, c->stream);
         std::vector<uint64_t> cnt(gidx.size());
         eis_stats st{};
         if (rc == EIS_OK) rc = plan_counts_user(p, cnt.data());
         if (rc == EIS_OK) rc = plan_fill_stats(p, &st);
-        plan_free(p);
+        plan_free(p, rc == EIS_OK);
         if (rc != EIS_OK) return rc;
         for (size_t k = 0; k < gidx.size(); ++k) counts_out[gidx[k]] = cnt[k];
         acc.candidates += st.candidates;
