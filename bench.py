@@ -59,12 +59,13 @@ TOP = 10**11
 # two subtractions, the multiply-add of the Q recurrence, two for the Z/3
 # class, two compares for the centre test and two for loop and exit
 OPS_PER_BABY_STEP = 11
-# int32-equivalent operations of one giant step of the lane search (the lean
-# product reduce(mu * G')): an extended Euclid on ~22-bit norms (about 13
-# division steps of quotient, remainder and two cofactor updates, 6 ops
-# each), three residue products (12), the product's assembly (6), the exact
-# division for Q_{-1} (10) and about three reduction steps (11 each)
-OPS_PER_GIANT_STEP = 140
+# int32-equivalent operations of one giant step of the lane search
+# (reduce(mu * Y), reduced while it is formed): nearest-integer Euclid on
+# ~21-bit norms (9 division steps of quotient, remainder and cofactor, 3 ops
+# each), the residue (4), the remainders down to d^(1/4) with both cofactors (5
+# steps of 4), four exact quotients (16), the form (12), its class (10),
+# normalisation (6) and one reduction step (11)
+OPS_PER_GIANT_STEP = 106
 SMS, LANES, SM_MAX_MHZ = 152, 128, 2070.0
 # offered request rates of the serving leg (req/s) and the cap on requests per rate
 SERVE_RATES = (10.0, 100.0, 1000.0, 3000.0, 10000.0, 30000.0, 100000.0)
@@ -141,7 +142,7 @@ class ClockSampler:
 KERNEL_SOURCES = {
     "k_walk_persistent": ("k_walk.cu", "eis_common.cuh"),
     "k_walk_record": ("k_bsgs.cu", "eis_bsgs.cuh", "eis_common.cuh"),
-    "k_bsgs_t": ("k_bsgs.cu", "eis_bsgs.cuh", "eis_infra.cuh", "eis_common.cuh"),
+    "k_bsgs_t": ("k_bsgs.cu", "eis_nuc.cuh", "eis_bsgs.cuh", "eis_infra.cuh", "eis_common.cuh"),
 }
 
 
@@ -326,14 +327,16 @@ def main():
     clocks = sampler.stop()
     count = int(plan.counts()[0])
     if tuned is not None:
-        mode_label = ("persistent work-stealing recording walk + lane-per-d infrastructure "
+        mode_label = ("cubic forms of discriminant d and 4d decide most d; the rest by the "
+                      "persistent work-stealing recording walk + lane-per-d infrastructure "
                       "search per decade (autotuned), CUDA graph")
     elif args.nbaby > 0:
         mode_label = ("persistent work-stealing recording walk + lane-per-d infrastructure "
                       "search after %d baby steps, 1 state in %d marked (set by hand), CUDA graph"
                       % (args.nbaby, args.mark_every))
     else:
-        mode_label = "persistent work-stealing walk of every d to its centre, CUDA graph"
+        mode_label = ("cubic forms of discriminant d and 4d decide most d; the rest by the "
+                      "recording walk + lane search at the library's own settings, CUDA graph")
     ms_step = sum(s["ms_total"] for s in sts) / len(sts)
     ms_walk = sum(s["ms_walk"] for s in sts) / len(sts)
     ms_giant = sum(s["ms_giant"] for s in sts) / len(sts)
@@ -374,7 +377,9 @@ def main():
         saved = ctx.tune_table()
         ctx.set_tune_table([])
         thr = ctx.get_option(E.EIS_OPT_GIANT_THRESHOLD)
+        lim = ctx.get_option(E.EIS_OPT_STEP_LIMIT)
         ctx.set_option(E.EIS_OPT_GIANT_THRESHOLD, 0)
+        ctx.set_option(E.EIS_OPT_STEP_LIMIT, 1 << 25)  # below its default: every d is walked
         wplan = ctx.plan_create([lo], [hi], E.EIS_MODE_PERSISTENT)
         one(wplan)
         wsts = [one(wplan) for _ in range(args.plain_steps)]
@@ -384,6 +389,7 @@ def main():
                      "baby_steps_per_step": wsts[0]["baby_steps"], "steps": args.plain_steps}
         wplan.destroy()
         ctx.set_option(E.EIS_OPT_GIANT_THRESHOLD, thr)
+        ctx.set_option(E.EIS_OPT_STEP_LIMIT, lim)
         ctx.set_tune_table(saved)
 
     # batched uneven ranges: 4096 seeded intervals in one persistent launch,
@@ -541,9 +547,9 @@ def main():
     e2e_s = sum(e2e_times) / len(e2e_times) if e2e_times else float("nan")
     ntiles = (n_cand + 65535) // 65536
     e2e = None if args.no_e2e else {"value": nD * world / e2e_s, "unit": UNIT,
-           "h2d_bytes_per_step": 24 + 16 * ntiles,   # interval + tile tables
-           "d2h_bytes_per_step": 2 * 4 * nw + 16 + 4 + 32,  # flag + square-free bitmaps, counts
-           "api": "eis_classify_range into pinned host buffers (plan build, graph capture, "
+           "h2d_bytes_per_step": 24 + 16 * ntiles + 2 * 48 + 1,  # interval, tile and form tables
+           "d2h_bytes_per_step": 2 * 4 * nw + 104,  # flag + square-free bitmaps, results
+           "api": "eis_classify_range into pinned host buffers (plan build, "
                   "device work, copies and sync inside the timed call; mean of 3 calls)"}
 
     peak = SMS * LANES * SM_MAX_MHZ * 1e6 / 1e9
@@ -589,6 +595,7 @@ def main():
                            "baby_steps_per_step": steps_per_launch,
                            "giant_steps_per_step": giant_per_launch,
                            "handed_to_search_per_step": sts[0]["deferred"],
+                           "ms_sieve_and_forms_per_step": sum(s["ms_sieve"] for s in sts) / len(sts),
                            "ms_walk_per_step": ms_walk, "ms_search_per_step": ms_giant,
                            "pi_E_window": count,
                            "l2": "flushed between steps (512 MiB write)",
