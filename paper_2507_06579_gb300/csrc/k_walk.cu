@@ -137,11 +137,19 @@ __device__ __forceinline__ void walk_persistent_body(
     uint32_t cand = 0;
     uint32_t done = 0;       // steps walked by the current d
     unsigned long long my_steps = 0;
+    uint32_t gap = 0;        // steps between the warp's centres, averaged
     for (;;) {
-        // Refill idle lanes; repeat while fresh d end at the first step.
+        // Refill idle lanes; repeat while fresh d end at the first step.  A
+        // refill costs about 200 instructions and the queue's latency for
+        // however many lanes take part, an idle lane 1/32 of the walk: lanes
+        // wait for one another while sqrt(985 / gap) is above their number
+        // (periods of a few hundred steps), never on long walks.  [5, 10^9]:
+        // walks of 670 steps on average, 5.2 ms a pass against 6.8.
+        const int batch = gap < 24 ? 6 : gap < 48 ? 4 : gap < 110 ? 3 : gap < 400 ? 2 : 1;
         for (;;) {
             const unsigned need = __ballot_sync(kFull, !active);
             if (need == 0 || exhausted) break;
+            if (__popc(need) < batch && need != kFull) break;
             const int leader = __ffs(need) - 1;
             uint32_t base = 0;
             if (lane == leader) base = atomicAdd(next_ptr, (uint32_t)__popc(need));
@@ -219,6 +227,7 @@ __device__ __forceinline__ void walk_persistent_body(
             }
             if (n >= room) break;
         }
+        gap = (3 * gap + min(n, 4096u)) >> 2;
         if (active) {
             done += n - back;
             if (hit) {
