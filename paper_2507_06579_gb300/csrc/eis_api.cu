@@ -326,11 +326,6 @@ static constexpr int64_t kCubicMinStepLimit = (int64_t)1 << 26;
 // about 15 us of the whole GPU, the cost of their launches).
 static constexpr double kCubicMinGain = 4e8;
 
-// Survivors a round of the lane search holds when the settings are the
-// library's own: 4.3 GB of tables (a smaller pool than the option's default
-// for callers who never asked for the search).
-static constexpr int64_t kAutoChunk = (int64_t)1 << 21;
-
 // The lane search's own settings: baby steps N = coef d^(1/4) and about 56
 // marked states, by d in steps of 4.  Measured best N (time flat within 3% for
 // N / 1.5 .. 1.5 N): of all d 768 / 1024..1536 / 2048 / 3072..6144 near 10^10 /
@@ -445,7 +440,7 @@ static int plan_enqueue(eis_plan *p, cudaStream_t s, bool capturing) {
                         p->d_glog, p->d_steps, p->d_status, limit, 0u, nullptr, nullptr, 0u,
                         p->fast);
                     record(p->bev[3 * r + 2], s, capturing);
-                    launches += 3;
+                    launches += 4;
                 }
             } else {
                 k_walk_persistent<<<p->walk_grid, 256, 0, s>>>(
@@ -677,8 +672,11 @@ static int plan_build(eis_ctx *c, const uint64_t *lo, const uint64_t *hi, size_t
         const uint64_t cached = pool_cached_bytes(c);  // reclaimable
         const uint64_t room = c->budget + cached > used + field_bytes ? c->budget + cached - used - field_bytes : 0;
         const uint64_t fit = room / per_d > lanes + 64 ? room / per_d - lanes - 64 : 0;
-        uint64_t C = std::min<uint64_t>((uint64_t)(own ? std::min(c->bsgs_chunk, kAutoChunk) : c->bsgs_chunk),
-                                        queue);
+        uint64_t C = std::min<uint64_t>((uint64_t)c->bsgs_chunk, queue);
+        // (for callers who never asked for the search its tables take a
+        // sixteenth of the budget at most; a round's tail, lanes that finish
+        // the longest searches alone, is 0.3 ms)
+        if (own) C = std::min<uint64_t>(C, c->budget / 16 / per_d / 32 * 32);
         C = std::min<uint64_t>(C, fit / 32 * 32);
         if (C >= ((uint64_t)1 << 16) || C >= queue) {
             p->bsgs = 1;

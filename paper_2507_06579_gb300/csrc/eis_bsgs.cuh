@@ -80,12 +80,21 @@ struct DEntry {
     uint32_t pad;
 };
 
-// A deferred d handed from the baby walk to the giant-step kernel.
+// A deferred d handed from the baby walk to the giant-step kernel: the walk
+// writes the first four words, k_prep the rest, all that the search starts
+// from (one thread a d there; a search lane is refilled alone).
 struct DRecord {
-    uint32_t cand;    // candidate index in the plan layout
-    uint32_t k;       // entries in the table (entry k-1 is G = a_jl)
-    uint32_t region;  // table region index in the pool
-    uint32_t s;       // floor(sqrt d)
+    uint32_t cand;           // candidate index in the plan layout
+    uint32_t k;              // entries in the table (entry k-1 is a_jl)
+    uint32_t region;         // table region index in the pool
+    int32_t s;               // floor(sqrt d)
+    int32_t Ma, Mb, Mg, Mw;  // where the search starts, its class and (b^2 - d)/(4a)
+    int32_t Ya, Yb, Yg, Yw;  // the stride
+    int32_t landed;          // 1: M = reduce(a_jl a_j') and Y is the same a few steps
+                             // on; 0: M = Y = a_jl, no product taken
+    int32_t L;               // floor(sqrt s)
+    float T;                 // marking threshold
+    uint32_t pad;
 };
 
 EIS_HD uint32_t float_bits(float f) {

@@ -64,8 +64,8 @@ __global__ void k_walk_record(const Seg *segs, uint32_t nseg, const uint32_t *su
                               const __grid_constant__ TuneTab tt, DRecord *recs, uint32_t *nrec,
                               uint32_t rec_cap, unsigned char *pool,
                               unsigned long long *handed_acc, int fast);
-// The lane search kernel for (fast quotient, composition), and its launch
-// (128 threads a block).
+// The lane search kernel for (fast quotient, composition), and the launch of
+// k_prep and of it (128 threads a block).
 const void *k_bsgs_kernel(int fast, int compose);
 cudaError_t launch_k_bsgs(uint32_t grid, cudaStream_t st, int fast, int compose, const Seg *segs,
                           uint32_t nseg, const DRecord *recs, const uint32_t *nrec, uint32_t rec_cap,

@@ -21,6 +21,8 @@
 //                 A d the search cannot finish (reduction or walk past its
 //                 limits) goes to a fallback list that the plain persistent
 //                 walk finishes.
+#include <algorithm>
+
 #include "eis.h"
 #include "eis_bsgs.cuh"
 #include "eis_common.cuh"
@@ -203,8 +205,8 @@ __device__ __forceinline__ void walk_record_body(
                     const uint32_t slot = atomicAdd(nrec, 1u);
                     if (slot < rec_cap) {
                         // s = floor(sqrt d) from C = 2s (+1), exactly
-                        const uint32_t sv = (uint32_t)__fmul_rn(kFast ? __fsub_rn(C, 1.0f) : C, 0.5f);
-                        *reinterpret_cast<uint4 *>(recs + slot) = make_uint4(cand, k, region, sv);
+                        const int32_t sv = (int32_t)__fmul_rn(kFast ? __fsub_rn(C, 1.0f) : C, 0.5f);
+                        *reinterpret_cast<uint4 *>(recs + slot) = make_uint4(cand, k, region, (uint32_t)sv);
                         // regions 0 .. lanes-1 are the lanes' first ones;
                         // region lanes + slot belongs to record slot `slot`,
                         // whose d has just left its region: the lane takes it
@@ -251,6 +253,63 @@ __global__ void __launch_bounds__(256, 3) k_walk_record(
         walk_record_body<false>(segs, nseg, surv, n_surv_ptr, q_lo, q_hi, next_ptr, flags, glog,
                                 steps_acc, status, step_limit, tt, recs, nrec, rec_cap, pool,
                                 handed_acc);
+}
+
+namespace {
+
+__device__ __forceinline__ NucIdeal entry_ideal(const uint4 &e, int32_t s, int64_t d) {
+    NucIdeal x;
+    x.a = (int32_t)__uint_as_float(e.x) / 2;
+    x.b = (int32_t)__uint_as_float(e.y) - s;  // floor(P + s (+ 1/2)) - s = P
+    x.g = (int32_t)(e.z % 3u);
+    x.w = nuc_w(x.a, x.b, d);
+    return x;
+}
+
+}  // namespace
+
+// Where each record's search starts and its stride, reduce(a_jl a_j') moved to
+// a norm without small factors, one thread a record.  (Done by the search's
+// lanes as they are refilled, two or three of 32 at a time, this was a quarter
+// of the search's instructions; at the hand-off in the recording walk, about 8
+// lanes at a time, it cost there what it saved here.)
+__global__ void __launch_bounds__(128) k_prep(const Seg *__restrict__ segs, uint32_t nseg,
+                                              DRecord *__restrict__ recs,
+                                              const uint32_t *__restrict__ nrec, uint32_t rec_cap,
+                                              const unsigned char *__restrict__ pool,
+                                              const __grid_constant__ TuneTab tt) {
+    const uint32_t n = min(*nrec, rec_cap);
+    for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+        uint4 *r = reinterpret_cast<uint4 *>(recs + i);
+        const uint4 r0 = r[0];  // cand, k, region, s
+        const uint4 *e = reinterpret_cast<const uint4 *>(pool + (size_t)r0.z * kBsgsRegionBytes);
+        const int32_t s = (int32_t)r0.w;
+        const int64_t d = (int64_t)cand_to_d(segs, nseg, r0.x);
+        const uint4 ge = e[r0.y - 1];
+        // j' = the last entry (not entry 0, not jl itself) at least kBsgsWideGap
+        // steps before jl
+        uint32_t ej = r0.y - 1;
+        do --ej; while (ej > 0 && e[ej].w + kBsgsWideGap > ge.w);
+        const int32_t L = (int32_t)isqrt44((uint64_t)s);
+        const NucIdeal G = entry_ideal(ge, s, d);
+        NucIdeal M = G, Y = G;
+        int st = kNucRetry;
+        if (ej > 0) {
+            const NucIdeal J = entry_ideal(e[ej], s, d);
+            NucIdeal x = G;
+            // a common factor: one step on (few d need more than two; one without
+            // the wide stride would take twice the giant steps)
+            for (int t = 0; t < 24 && st == kNucRetry; ++t) {
+                if (t) x = nuc_step(x, s);
+                st = nuc_mul(x, J, s, L, M);
+            }
+            if (st == kNucOk) Y = nuc_coprime(M, s); else M = G;
+        }
+        const float T = __fmul_rn(tt.tau[tune_row(tt, (uint64_t)d)], __uint2float_rn((uint32_t)s));
+        r[1] = make_uint4((uint32_t)M.a, (uint32_t)M.b, (uint32_t)M.g, (uint32_t)M.w);
+        r[2] = make_uint4((uint32_t)Y.a, (uint32_t)Y.b, (uint32_t)Y.g, (uint32_t)Y.w);
+        r[3] = make_uint4(st == kNucOk, (uint32_t)L, __float_as_uint(T), 0u);
+    }
 }
 
 namespace {
@@ -312,14 +371,10 @@ __device__ __forceinline__ void bsgs_body(
     int32_t s = 0, L = 0;  // floor(sqrt d) < 2^22 and its square root
     float T = 0.0f, C = 0.0f;
     const uint4 *tab = nullptr;
-    // G = a_jl starts the search; the stride Y is reduce(a_jl * a_j') (taken
-    // by the first cycle from Y = a_j', `first`), or a_jl when no table state
-    // lies kBsgsWideGap steps before jl
-    // reduced ideals of the lane's d, every coefficient below 2^22: held in
-    // 32 bits and widened for the product
-    SIdeal G{1, 1, 0}, mu{1, 1, 0}, Y{1, 1, 0};
+    // mu and the stride Y = reduce(a_jl * a_j') (or a_jl), from the record
+    SIdeal mu{1, 1, 0}, Y{1, 1, 0};
     int32_t wY = 0, wmu = 0;  // third form coefficients (b^2 - d)/(4a) of Y and mu
-    bool first = false;
+    bool landed = false;  // mu is a product: its walk begins
     // the lane's walk, carried across iterations: it composes when its last
     // walk has ended (compose_now), else walks on
     LeanState w;
@@ -343,12 +398,24 @@ __device__ __forceinline__ void bsgs_body(
             if (!active) {
                 const uint32_t idx = base + __popc(need & lt);
                 if (idx < n) {
-                    const uint4 r0 = *reinterpret_cast<const uint4 *>(recs + idx);  // cand, k, region, s
+                    const uint4 *r = reinterpret_cast<const uint4 *>(recs + idx);
+                    const uint4 r0 = r[0], r1 = r[1], r2 = r[2], r3 = r[3];
                     cand = r0.x;
                     k = r0.y;
                     tab = reinterpret_cast<const uint4 *>(pool + (size_t)r0.z * kBsgsRegionBytes);
                     s = (int32_t)r0.w;
-                    fresh = true;
+                    mu = SIdeal{(int32_t)r1.x, (int32_t)r1.y, (int32_t)r1.z};
+                    wmu = (int32_t)r1.w;
+                    Y = SIdeal{(int32_t)r2.x, (int32_t)r2.y, (int32_t)r2.z};
+                    wY = (int32_t)r2.w;
+                    landed = r3.x != 0;  // its first product is taken: walk on from it
+                    compose_now = !landed;
+                    cycles = landed;
+                    L = (int32_t)r3.y;
+                    T = __uint_as_float(r3.z);
+                    C = __uint2float_rn((uint32_t)(kFast ? 2 * s + 1 : 2 * s));
+                    if (kCompose == 1) d = (int64_t)cand_to_d(segs, nseg, cand);
+                    active = fresh = true;
                 }
             }
         }
@@ -362,86 +429,20 @@ __device__ __forceinline__ void bsgs_body(
             const uint4 *e = reinterpret_cast<const uint4 *>(
                 __shfl_sync(kFull, reinterpret_cast<unsigned long long>(tab), src));
             uint32_t *sl = fp_warp + src * kFpWords;
-            uint4 v[kBsgsKmax / 32];
+            uint32_t q[kBsgsKmax / 32];  // (all loads in flight at once)
 #pragma unroll
-            for (int t = 0; t < kBsgsKmax / 32; ++t) {
-                const uint32_t i = lane + 32 * t;
-                v[t] = i < kk ? e[i] : make_uint4(0u, 0u, 0u, 0u);
-            }
+            for (int t = 0; t < kBsgsKmax / 32; ++t)
+                if (lane + 32 * t < kk) q[t] = e[lane + 32 * t].x;
             sl[lane] = 0u;
             __syncwarp();
 #pragma unroll
             for (int t = 0; t < kBsgsKmax / 32; ++t)
                 if (lane + 32 * t < kk) {
                     uint32_t word, mask;
-                    fp_bits(v[t].x, word, mask);
+                    fp_bits(q[t], word, mask);
                     atomicOr(&sl[word], mask);
                 }
-            // G = entry kk-1, held by lane (kk-1) % 32 in v[(kk-1) / 32]
-            const uint32_t tg = (kk - 1) >> 5;
-            uint32_t gx = 0, gy = 0, gz = 0;
-#pragma unroll
-            for (int t = 0; t < kBsgsKmax / 32; ++t) {
-                if ((uint32_t)t == tg) {
-                    gx = v[t].x;
-                    gy = v[t].y;
-                    gz = v[t].z;
-                }
-            }
-            gx = __shfl_sync(kFull, gx, (kk - 1) & 31);
-            gy = __shfl_sync(kFull, gy, (kk - 1) & 31);
-            gz = __shfl_sync(kFull, gz, (kk - 1) & 31);
-            const uint32_t jlast = __shfl_sync(kFull, (tg == 0 ? v[0].w : tg == 1 ? v[1].w
-                                                       : tg == 2 ? v[2].w : v[3].w), (kk - 1) & 31);
-            // j' = the last entry (not entry 0, not jl itself) at least
-            // kBsgsWideGap steps before jl
-            uint32_t ej = 0;
-#pragma unroll
-            for (int t = 0; t < kBsgsKmax / 32; ++t) {
-                const uint32_t i = lane + 32 * t;
-                if (i >= 1 && i + 1 < kk && v[t].w + kBsgsWideGap <= jlast) ej = max(ej, i);
-            }
-            ej = __reduce_max_sync(kFull, ej);
-            const uint32_t tj = ej >> 5;
-            uint32_t jx = 0, jy = 0, jz = 0;
-#pragma unroll
-            for (int t = 0; t < kBsgsKmax / 32; ++t) {
-                if ((uint32_t)t == tj) {
-                    jx = v[t].x;
-                    jy = v[t].y;
-                    jz = v[t].z;
-                }
-            }
-            jx = __shfl_sync(kFull, jx, ej & 31);
-            jy = __shfl_sync(kFull, jy, ej & 31);
-            jz = __shfl_sync(kFull, jz, ej & 31);
-            if (lane == src) {
-                G.a = (int32_t)__uint_as_float(gx) / 2;
-                G.b = (int32_t)__uint_as_float(gy) - s;  // floor(P + s (+ 1/2)) - s = P
-                G.g = (int)(gz % 3u);
-                first = ej > 0;
-                if (first) {
-                    Y.a = (int32_t)__uint_as_float(jx) / 2;
-                    Y.b = (int32_t)__uint_as_float(jy) - s;
-                    Y.g = (int)(jz % 3u);
-                } else {
-                    Y = G;
-                }
-            }
             __syncwarp();
-        }
-        if (fresh) {
-            d = (int64_t)cand_to_d(segs, nseg, cand);
-            L = (int32_t)isqrt44((uint64_t)s);
-            wmu = nuc_w(G.a, G.b, d);
-            wY = nuc_w(Y.a, Y.b, d);
-            C = __uint2float_rn((uint32_t)(kFast ? 2 * s + 1 : 2 * s));
-            Cw = C;
-            T = __fmul_rn(tt.tau[tune_row(tt, (uint64_t)d)], __uint2float_rn((uint32_t)s));
-            mu = G;
-            cycles = 0;
-            active = true;
-            compose_now = true;
         }
         if (!__any_sync(kFull, active)) break;
         // ---- giant step for the lanes whose last walk has ended:
@@ -474,24 +475,21 @@ __device__ __forceinline__ void bsgs_body(
                 mu = SIdeal{m1.a, m1.b, m1.g};
                 wmu = m1.w;
             } else {
-                if (first) {
-                    // the first landing, reduce(a_jl * a_j'), is the stride (a
-                    // few steps on, at a norm without small factors)
-                    first = false;
-                    const NucIdeal y1 = kCompose == 0 ? nuc_coprime(nx, s) : nx;
-                    Y = SIdeal{y1.a, y1.b, y1.g};
-                    wY = y1.w;
-                }
-                Cw = C;  // (parked while the lane waited)
-                w.num = bsgs_num(nx.b, s, kFast);
-                w.Q = __uint2float_rn((uint32_t)(2 * nx.a));
-                w.Qp = __uint2float_rn((uint32_t)(-2 * nx.w));
-                w.x = (int)((nx.b >> 1) & 1);
-                w.acc = 0;
-                gc = nx.g;
-                walked = 0;
-                compose_now = false;
+                mu = SIdeal{nx.a, nx.b, nx.g};
+                wmu = nx.w;
+                landed = true;
             }
+        }
+        if (landed) {
+            landed = compose_now = false;
+            Cw = C;  // (parked while the lane waited)
+            w.num = bsgs_num(mu.b, s, kFast);
+            w.Q = __uint2float_rn((uint32_t)(2 * mu.a));
+            w.Qp = __uint2float_rn((uint32_t)(-2 * wmu));
+            w.x = (int)((mu.b >> 1) & 1);
+            w.acc = 0;
+            gc = mu.g;
+            walked = 0;
         }
         // ---- walk at most walk_window steps toward the first marked state x
         // and one step beyond; a walk that needs more goes on next iteration
@@ -547,33 +545,27 @@ __device__ __forceinline__ void bsgs_body(
                 __shfl_sync(kFull, reinterpret_cast<unsigned long long>(tab), src));
             const uint32_t sq = __shfl_sync(kFull, kq, src), sd = __shfl_sync(kFull, kd, src),
                            sm = __shfl_sync(kFull, km, src);
-            int jd = 0x7fffffff, jm = 0x7fffffff;
-            uint32_t Sd = 0, Sm = 0;
+            // positions are distinct states: at most one entry matches each key
+            uint4 v[kBsgsKmax / 32];
 #pragma unroll
-            for (int t = 0; t < kBsgsKmax / 32; ++t) {
-                const uint32_t i = lane + 32 * t;
-                if (i < kk) {
-                    const uint4 v = e[i];
-                    if (v.x == sq && v.y == sd && (int)i < jd) {
-                        jd = (int)i;
-                        Sd = v.z;
-                    }
-                    if (v.x == sq && v.y == sm && (int)i < jm) {
-                        jm = (int)i;
-                        Sm = v.z;
-                    }
+            for (int t = 0; t < kBsgsKmax / 32; ++t)
+                v[t] = lane + 32 * t < kk ? e[lane + 32 * t] : make_uint4(0u, 0u, 0u, 0u);
+            uint32_t S = 0;
+            bool hd = false, hm = false;
+#pragma unroll
+            for (int t = 0; t < kBsgsKmax / 32; ++t)
+                if (v[t].x == sq && (v[t].y == sd || v[t].y == sm)) {
+                    if (v[t].y == sd) hd = true; else hm = true;
+                    S = v[t].z;
                 }
-            }
-            const unsigned hd = __ballot_sync(kFull, jd != 0x7fffffff);
-            const unsigned hm = __ballot_sync(kFull, jm != 0x7fffffff);
-            const uint32_t Sd0 = __shfl_sync(kFull, Sd, hd ? __ffs(hd) - 1 : 0);
-            const uint32_t Sm0 = __shfl_sync(kFull, Sm, hm ? __ffs(hm) - 1 : 0);
-            if (lane == src) {
-                const int gx = gc - 1 - w.x;
-                if (hd)
-                    g = (gx - (int)(Sd0 % 3u) + 3 * 4) % 3;  // x = l + j
-                else if (hm)
-                    g = (gx + (int)(Sm0 % 3u)) % 3;          // x = l - j
+            const unsigned bd = __ballot_sync(kFull, hd), bm = __ballot_sync(kFull, hm);
+            if (bd | bm) {
+                S = __shfl_sync(kFull, S, __ffs(bd ? bd : bm) - 1) % 3u;
+                if (lane == src) {
+                    const int gx = gc - 1 - w.x;
+                    g = bd ? (gx - (int)S + 3 * 4) % 3   // x = l + j
+                           : (gx + (int)S) % 3;          // x = l - j
+                }
             }
         }
         if (!at_end) continue;
@@ -626,6 +618,9 @@ cudaError_t launch_k_bsgs(uint32_t grid, cudaStream_t st, int fast, int compose,
                           uint32_t *fb_count, uint32_t fb_cap, const TuneTab &tt,
                           uint32_t max_cycles, uint32_t walk_cap, uint32_t walk_window) {
     TuneTab t = tt;
+    k_prep<<<std::min(rec_cap / 128 + 1, 4 * grid), 128, 0, st>>>(
+        segs, nseg, const_cast<DRecord *>(recs), nrec, rec_cap, pool, tt);
+    if (cudaError_t e = cudaPeekAtLastError(); e != cudaSuccess) return e;
     void *args[] = {&segs, &nseg, &recs, &nrec, &rec_cap, &next_ptr, &pool, &flags, &glog,
                     &acc, &status, &fb_list, &fb_count, &fb_cap, &t, &max_cycles, &walk_cap,
                     &walk_window};
