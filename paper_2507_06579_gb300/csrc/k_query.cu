@@ -7,22 +7,24 @@
 //    rcp -> quotient -> remainder -> Q') stores each state with one shared
 //    store; the 8 warps insert the states afterwards, 2N / 256 rounds;
 //  * 256 lanes of giant steps let N be a quarter of what 32 lanes want;
-//  * lane t = 32 w + l holds mu = S^(t+1), S = reduce(a_N a_{N/2}): S^(l+1) by
-//    a scan over the lanes (5 products deep), H = S^32, H^w by another (3),
-//    and one product.  Later rounds multiply by H^8 = S^256.
+//  * thread t holds mu_t = S^(t+1), S = reduce(a_N a_{N/2}): once the first k
+//    = 1, 2, 4, .. 128 are known, threads k .. 2k - 1 take mu_{t-k} S^k, and a
+//    hit among them ends the search; after 256, rounds of mu_t S^256.
 // All products are nuc_mul (eis_nuc.cuh) in one out-of-line copy (the kernel
 // runs once, so its instructions come from L2).
 //
 // Coverage.  The table holds the window [R - delta_N, R + delta_N] whole
 // (every state, and its mirror).  S is shorter than the window by
 // delta_N - delta_{N/2}, at least N/4 pairs of steps of log 2 or more each;
-// two neighbouring powers differ by S up to the offsets of the (at most 9)
+// two neighbouring powers differ by S up to the offsets of the (at most 8)
 // products they do not share, each below log 2 sqrt d, and their few steps to
 // a norm without small factors.
 //
-// Measured, a call with its launch: 43 us against 161 us for d below 10^12, 63
+// Measured, a call with its launch: 39 us against 161 us for d below 10^12, 58
 // against 290 below 2^44 (one warp, table and giant steps alike); 75 and 102
-// with the textbook product, whose 1100 serial instructions are 5 us.
+// with the textbook product, whose 1100 serial instructions are 5 us; 43 and 60
+// with two scans over the lanes (10 products deep) instead of the doubling (9,
+// and 6 to 8 when a hit comes early).
 #include "eis_common.cuh"
 #include "eis_bsgs.cuh"
 #include "eis_infra.cuh"
@@ -32,8 +34,6 @@
 namespace eis {
 
 namespace {
-
-constexpr int kQWarps = kQueryThreads / 32;
 
 // Ideals as (a, b, class, w = (b^2 - d)/(4a)): reduce(X * Y), moved on to a
 // norm without small factors; a = 0 when a factor has failed or a reduction
@@ -127,6 +127,7 @@ __global__ void __launch_bounds__(kQueryThreads) k_query(uint64_t d, const uint6
     uint64_t *tab = smem_q;
     float4 *st = reinterpret_cast<float4 *>(smem_q + ((size_t)1 << log2n));  // N + 2 states
     __shared__ int sh_done, sh_g, sh_steps, sh_ok, sh_best[2];
+    __shared__ int4 sh_mu[kQueryThreads];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const bool fast = d < kFastDLimit;
     if (warp == 0) {
@@ -165,63 +166,75 @@ __global__ void __launch_bounds__(kQueryThreads) k_query(uint64_t d, const uint6
     }
     if (!ok) sh_ok = 0;
     __syncthreads();
-    // ---- S, then S^(l+1) on lane l (every warp alike)
+    // ---- powers of S: mu_t of thread t, doubled level by level, each looked up
+    // as it is made.  best: the first hit (-1: a product failed); two words in
+    // turn, so that a level or round that goes on leaves its word as it was.
     auto state = [&](int j) {
         const float4 x = st[j];
         return make_int4((int)x.x / 2, (int)x.y - s, (int)((uint32_t)__float_as_int(x.z) % 3u),
                          -(int)st[j - 1].x / 2);
     };
-    int4 mu = query_mul(state(N), state(N / 2), (int64_t)d, s, L);
-#pragma unroll 1
-    for (int k = 1; k < 32; k <<= 1) {
-        const int4 o = shfl4(mu, lane >= k ? lane - k : lane);
-        if (lane >= k) mu = query_mul(mu, o, (int64_t)d, s, L);
-    }
-    auto found = [&](uint64_t e) {  // log eps_d from the table's entry at mu
-        const int Sj = (int)(e & 3);
-        return (e & 4) ? (mu.z + Sj) % 3 : (mu.z + 3 - Sj) % 3;
+    int4 mu = make_int4(0, 0, 0, 0);
+    uint64_t e = 0;
+    auto look = [&](int word) {
+        e = mu.x ? infra_find(tab, log2n, infra_key(2 * (int64_t)mu.x, mu.y)) : 0;
+        if (!mu.x)
+            atomicMin(&sh_best[word], -1);
+        else if (e)
+            atomicMin(&sh_best[word], tid);
     };
-    if (!__all_sync(kFull, mu.x != 0)) sh_ok = 0;
-    uint64_t e = mu.x ? infra_find(tab, log2n, infra_key(2 * (int64_t)mu.x, mu.y)) : 0;
-    const unsigned early = __ballot_sync(kFull, e != 0);  // the same in every warp
-    __syncthreads();
-    if (early || !sh_ok) {
-        if (warp == 0 && lane == (early ? __ffs(early) - 1 : 0)) {
+    auto finish = [&](int best, uint32_t giants) {  // by every thread: best is decided
+        if (tid == max(best, 0)) {
+            const int Sj = (int)(e & 3);
             out->baby = 1 + (uint32_t)sh_steps;
-            out->giant = 6 + (uint32_t)lane;
-            out->result = sh_ok ? 1 + found(e) : -1;
+            out->giant = giants;
+            out->result = best < 0 ? -1 : 1 + ((e & 4) ? (mu.z + Sj) % 3 : (mu.z + 3 - Sj) % 3);
         }
+    };
+    if (warp == 0) {
+        // the first 32 in one warp, by shuffles
+        if (lane == 0) mu = query_mul(state(N), state(N / 2), (int64_t)d, s, L);
+        __syncwarp();
+#pragma unroll 1
+        for (int k = 1; k < 32; k <<= 1) {
+            const int4 o = shfl4(mu, lane & (k - 1)), P = shfl4(mu, k - 1);
+            if (lane >= k && lane < 2 * k) mu = query_mul(o, P, (int64_t)d, s, L);
+        }
+        look(0);
+        sh_mu[lane] = mu;
+    }
+    __syncthreads();
+    if (sh_best[0] < kQueryThreads || !sh_ok) {
+        finish(sh_ok ? sh_best[0] : -1, 6u + (uint32_t)tid);
         return;
     }
-    // ---- H = S^32; lane i: H^(i+1); mu = S^(l+1) H^w, the stride H^8
-    int4 h = shfl4(mu, 31);
+    int word = 1;
 #pragma unroll 1
-    for (int k = 1; k < kQWarps; k <<= 1) {
-        const int4 o = shfl4(h, lane >= k ? lane - k : lane);
-        if (lane >= k && lane < kQWarps) h = query_mul(h, o, (int64_t)d, s, L);
-    }
-    const int4 stride = shfl4(h, kQWarps - 1);
-    const int4 hw = shfl4(h, warp > 0 ? warp - 1 : 0);
-    if (warp > 0) mu = query_mul(mu, hw, (int64_t)d, s, L);
-    for (uint32_t r = 0; r < max_rounds; ++r) {
-        // the first hit of the round; -1: a product failed.  (Two words in turn:
-        // a round that goes on leaves its word as it was.)
-        e = mu.x ? infra_find(tab, log2n, infra_key(2 * (int64_t)mu.x, mu.y)) : 0;
-        if (!mu.x || !stride.x)
-            atomicMin(&sh_best[r & 1], -1);
-        else if (e)
-            atomicMin(&sh_best[r & 1], tid);
+    for (int k = 32; k < kQueryThreads; k <<= 1) {
+        if (tid >= k && tid < 2 * k) {
+            mu = query_mul(sh_mu[tid - k], sh_mu[k - 1], (int64_t)d, s, L);
+            look(word);
+            sh_mu[tid] = mu;
+        }
         __syncthreads();
-        const int best = sh_best[r & 1];
+        const int best = sh_best[word];
         if (best < kQueryThreads) {
-            if (tid == max(best, 0)) {
-                out->baby = 1 + (uint32_t)sh_steps;
-                out->giant = 10 + kQueryThreads * r + (uint32_t)tid;
-                out->result = best >= 0 ? 1 + found(e) : -1;
-            }
+            finish(best, 6u + (uint32_t)tid);
             return;
         }
+        word ^= 1;
+    }
+    const int4 stride = sh_mu[kQueryThreads - 1];
+    for (uint32_t r = 1; r < max_rounds; ++r) {
         mu = query_mul(mu, stride, (int64_t)d, s, L);
+        look(word);
+        __syncthreads();
+        const int best = sh_best[word];
+        if (best < kQueryThreads) {
+            finish(best, 6u + kQueryThreads * r + (uint32_t)tid);
+            return;
+        }
+        word ^= 1;
     }
     if (tid == 0) out->result = -1;  // no hit within max_rounds
 }
