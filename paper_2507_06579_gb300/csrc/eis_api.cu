@@ -362,19 +362,19 @@ static bool tune_rows(const eis_ctx *c, TuneTab &tt) {
 
 // What the cubic forms save on a segment, in thread instructions (negative:
 // they cost more).  A walk takes about 0.067 sqrt(d) steps of 13.3
-// instructions, with the lane search about 16.7 d^(1/4) steps' worth (3.1 ns a
+// instructions, with the lane search about 14.5 d^(1/4) steps' worth (2.7 ns a
 // d near 10^11); the forms save 0.9 of that (with a log output, where they
 // decide only d in E, 0.29).  The enumeration looks at about 0.135 d^(3/4)
 // triples for kind 0 and 0.057 d^(3/4) for kind 1, whatever the window's width
-// (counted at 10^9 .. 2^44), at about 500 instruction slots each.
+// (counted at 10^9 .. 2^44), at about 250 instruction slots each.
 static double cubic_gain(const Seg &s, bool search, bool with_log, bool primes) {
     if (s.ncand == 0) return -1.0;
     const double d = (double)(s.d0 + 8 * (s.ncand - 1));
     double steps = 0.067 * std::sqrt(d);
-    if (search) steps = std::min(steps, 16.7 * std::sqrt(std::sqrt(d)));
+    if (search) steps = std::min(steps, 14.5 * std::sqrt(std::sqrt(d)));
     const double density = primes ? 4.0 / std::log(d) : 0.81;
     const double walk = (double)s.ncand * density * steps * 13.3 * (with_log ? 0.29 : 0.9);
-    const double forms = 500.0 * std::pow(d, 0.75) * (with_log ? 0.135 : 0.192);
+    const double forms = 250.0 * std::pow(d, 0.75) * (with_log ? 0.135 : 0.192);
     return 0.8 * walk - forms;
 }
 

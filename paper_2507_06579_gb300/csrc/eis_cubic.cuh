@@ -68,17 +68,20 @@ struct CubicJob {
     uint32_t amax;    // a = 1 .. amax
     uint32_t nblk;    // blocks of kCubicBlock b's: b < nblk * kCubicBlock
     uint32_t unit0;   // first unit of the job in the launch's numbering
+    uint32_t slices;  // slices of a unit at a = 1
+    uint32_t pad;
 };
 
-// Slices a unit (a; 16 b's) is cut into: the forms of a window thin out like
-// 1/a^2, and a slice takes every S-th of 32 forms.
-EIS_HD uint32_t cubic_slices(uint32_t a) { return a < 8 ? 64u / (a * a) : 1u; }
+// Slices a unit (a; 16 b's) is cut into, of s1 at a = 1: the forms of a window
+// thin out like 1/a^2, and a slice takes every S-th of 32 forms (but looks at
+// every c, so that narrow windows have s1 = 1).
+EIS_HD uint32_t cubic_slices(uint32_t a, uint32_t s1) { return a * a < s1 ? s1 / (a * a) : 1u; }
 
-// Units of a's below `a` (per block of b's): sum of cubic_slices.
-EIS_HD uint32_t cubic_slices_below(uint32_t a) {
+// Units of a's below `a` (per block of b's): sum of cubic_slices (s1 <= 64).
+EIS_HD uint32_t cubic_slices_below(uint32_t a, uint32_t s1) {
     uint32_t n = a > 8 ? a - 8 : 0u;
     const uint32_t m = a < 8 ? a : 8u;
-    for (uint32_t i = 1; i < m; ++i) n += cubic_slices(i);
+    for (uint32_t i = 1; i < m; ++i) n += cubic_slices(i, s1);
     return n;
 }
 
@@ -101,12 +104,21 @@ EIS_HD float cubic_sqrt(float x) {
 #endif
 }
 
-// x y rounded to an integer next to it, |x y| < 2^22.
-EIS_HD int32_t cubic_rint(float x, float y) {
+// 1.5 2^23 + x y rounded to an integer, |x y| < 2^22: its low bits are the
+// integer's.
+EIS_HD float cubic_rint(float x, float y) {
 #ifdef __CUDA_ARCH__
-    return __float_as_int(__fmaf_rn(x, y, 12582912.0f)) - 0x4B400000;
+    return __fmaf_rn(x, y, 12582912.0f);
 #else
-    return (int32_t)float_bits(std::fma(x, y, 12582912.0f)) - 0x4B400000;
+    return std::fma(x, y, 12582912.0f);
+#endif
+}
+
+EIS_HD float cubic_fma(float x, float y, float z) {
+#ifdef __CUDA_ARCH__
+    return __fmaf_rn(x, y, z);
+#else
+    return std::fma(x, y, z);
 #endif
 }
 
@@ -156,7 +168,8 @@ EIS_HD int32_t cubic_floordiv(int32_t x, int32_t m, float rm, int32_t &rem) {
 // Constants of a job for one a.
 struct CubicA {
     int32_t a, kind;
-    int64_t K0, K1;   // 9a disc at the window's ends
+    float K0h, K0l;   // 9a disc at the window's least end, in two floats
+    float dK;         // ... and what it grows by to the other
     float k0, k1;     // 27 a^2 disc / 4 there
     float pmax;       // sqrt of the largest discriminant, widened
     float r9a, r3a;   // 1/(9a), 1/(3a)
@@ -168,11 +181,13 @@ EIS_HD CubicA cubic_a(const CubicJob &j, int32_t a) {
     const int64_t D0 = m * (int64_t)j.d0, D1 = m * (int64_t)(j.d0 + 8 * (j.ncand - 1));
     A.a = a;
     A.kind = (int32_t)j.kind;
-    A.K0 = 9 * a * D0;  // < 9 * 1115 * 2^46
-    A.K1 = 9 * a * D1;
+    const int64_t K0 = 9 * a * D0, K1 = 9 * a * D1;  // < 9 * 1115 * 2^46
+    A.K0h = (float)K0;
+    A.K0l = (float)(K0 - (int64_t)A.K0h);
+    A.dK = (float)(K1 - K0);
     const float s = 0.75f * (float)a;
-    A.k0 = s * (float)A.K0;
-    A.k1 = s * (float)A.K1;
+    A.k0 = s * A.K0h;
+    A.k1 = s * (float)K1;
     A.pmax = cubic_sqrt((float)D1) * 1.000001f + 1.0f;
     A.r9a = 1.0f / (9.0f * (float)a);
     A.r3a = 1.0f / (3.0f * (float)a);
@@ -214,10 +229,9 @@ EIS_HD int32_t cubic_c_range(const CubicA &A, int32_t b, float plo, float phi, i
     return c1 >= c0 ? (c1 - c0) / 2 + 1 : 0;
 }
 
-// The forms of one (a, b, c): Q = rho + 9a k, e = e0 - k.  Two bands of k,
+// The forms of one (a, b, c): Q = rho + 9a k.  Two bands of k,
 // k = k[i] + (t << cubic_shift) for 0 <= t < n[i].
 struct CubicBands {
-    int32_t P, rho, e0;
     int32_t k[2], n[2];
 };
 
@@ -225,29 +239,36 @@ struct CubicBands {
 // mod 4.
 EIS_HD int32_t cubic_shift(int kind, int32_t a) { return (!kind && (a & 1)) ? 2 : 1; }
 
-EIS_HD void cubic_one_band(const CubicA &A, float qlo, float qhi, float P, int32_t rho, int32_t kres,
-                           int32_t sh, int32_t &k0, int32_t &n) {
-    const float m = 1.0f + 2.5e-6f * P + (float)rho;
-    const int32_t lo = cubic_ceil((fmaxf(qlo, -1.0f) * P - m) * A.r9a);
-    const int32_t hi = cubic_floor((fminf(qhi, 1.0f) * P + (m - 2.0f * (float)rho)) * A.r9a);
+// bc = 9a e0 + rho with rho small, e = e0 - k: rho, and the roundings that
+// make up e0 = b cq + q2 (as cubic_rint's floats).
+EIS_HD float cubic_rho(const CubicA &A, float fb, float fc, float &cq, float &q2) {
+    const float m9a = 9.0f * (float)A.a;
+    cq = cubic_rint(fc, A.r9a);
+    const float bc0 = fb * cubic_fma(-m9a, cq - 12582912.0f, fc);  // exact, below 2^24
+    q2 = cubic_rint(bc0, A.r9a);
+    return cubic_fma(-m9a, q2 - 12582912.0f, bc0);
+}
+
+// Forms of a band qlo <= q <= qhi: its first k and their number.
+EIS_HD void cubic_one_band(const CubicA &A, float qlo, float qhi, float P, float mlo, float mhi,
+                           int32_t kres, int32_t sh, int32_t &k0, int32_t &n) {
+    const int32_t lo = cubic_ceil((fmaxf(qlo, -1.0f) * P - mlo) * A.r9a);
+    const int32_t hi = cubic_floor((fminf(qhi, 1.0f) * P + mhi) * A.r9a);
     k0 = lo + ((kres - lo) & ((1 << sh) - 1));
     n = hi >= k0 ? ((hi - k0) >> sh) + 1 : 0;
 }
 
-EIS_HD void cubic_bands(const CubicA &A, int32_t b, int32_t c, CubicBands &B) {
+// Everything here is fp32: b, c and P are integers below 2^24, and
+// n = 4c + 9a disc / P^2, which cancels, is formed from 9a disc and P^2 in two
+// floats each, one step of Newton on the quotient.
+EIS_HD CubicBands cubic_bands(const CubicA &A, int32_t b, int32_t c) {
+    CubicBands B;
+    B.n[0] = B.n[1] = B.k[0] = B.k[1] = 0;
     const int32_t a = A.a;
-    const int32_t P = b * b - 3 * a * c;
-    B.P = P;
-    B.n[0] = B.n[1] = 0;
-    B.k[0] = B.k[1] = 0;
-    B.rho = B.e0 = 0;
-    if (P < 1) return;
-    // bc = 9a e0 + rho, rho small (e0 mod 2^32 is enough)
-    const int32_t cq = cubic_rint((float)c, A.r9a), c0 = c - 9 * a * cq;
-    const int32_t q2 = cubic_rint((float)(b * c0), A.r9a);
-    const int32_t rho = b * c0 - 9 * a * q2;
-    B.e0 = b * cq + q2;
-    B.rho = rho;
+    const float fb1 = (float)b, fc = (float)c, fa = 3.0f * (float)a;
+    const float P = cubic_fma(-fa, fc, fb1 * fb1);  // >= 1 (cubic_c_range)
+    float cq, q2;
+    const float rho = cubic_rho(A, fb1, fc, cq, q2);
     // e == er mod the step  <=>  k == e0 - er
     const int32_t sh = cubic_shift(A.kind, a);
     int32_t er;
@@ -255,38 +276,45 @@ EIS_HD void cubic_bands(const CubicA &A, int32_t b, int32_t c, CubicBands &B) {
         er = (a & b & 1) ? 0 : 1;
     else
         er = !(a & 1) ? 1 : (b & 1) ? 2 - a - b - c : 2;
-    const int32_t kres = B.e0 - er;
+    const int32_t kres = b * (int32_t)float_bits(cq) + (int32_t)float_bits(q2) - er;
     // h(q) between n0 and n1; u = sqrt(4b^2 - 3a n) at either end, on the side
     // that widens n / (2b + u)
-    const float fP = (float)P, rP2 = cubic_rcp(fP * fP);
-    const int64_t cP2 = 4 * (int64_t)c * ((int64_t)P * P);
-    const float n0 = (float)(A.K0 + cP2) * rP2, n1 = (float)(A.K1 + cP2) * rP2;
-    const float fb = 2.0f * (float)b, fa = 3.0f * (float)a, fb2 = fb * fb;
-    const float t0 = fb2 - fa * n0, t1 = fb2 - fa * n1;
-    const float e0 = 1e-6f * (fb2 + fa * fabsf(n0)), e1 = 1e-6f * (fb2 + fa * fabsf(n1));
-    if (t0 + e0 < 0.0f) return;  // the window lies above the largest h
-    const float ua = cubic_sqrt(fmaxf(n0 >= 0.0f ? t0 + e0 : t0 - e0, 0.0f));
-    const float ub = cubic_sqrt(fmaxf(n1 >= 0.0f ? t1 - e1 : t1 + e1, 0.0f));
+    const float ph = P * P, pl = cubic_fma(P, P, -ph), rp = cubic_rcp(ph);
+    const float z = A.K0h * rp;
+    const float zc = (cubic_fma(-z, ph, A.K0h) + cubic_fma(-z, pl, A.K0l)) * rp;
+    const float n0 = cubic_fma(4.0f, fc, z) + zc, n1 = cubic_fma(A.dK, rp, n0);
+    const float fb = 2.0f * fb1, fb2 = fb * fb;
+    const float t0 = cubic_fma(-fa, n0, fb2), t1 = cubic_fma(-fa, n1, fb2);
+    // 1e-6 (4b^2 + 3a |n|) at the larger of the two
+    const float e = 1e-6f * (2.0f * fb2 + fmaxf(fabsf(t0), fabsf(t1)));
+    if (t0 + e < 0.0f) return B;  // the window lies above the largest h
+    const float ua = cubic_sqrt(fmaxf(n0 >= 0.0f ? t0 + e : t0 - e, 0.0f));
+    const float ub = cubic_sqrt(fmaxf(n1 >= 0.0f ? t1 - e : t1 + e, 0.0f));
     const float qs = fb * A.r3a;  // q*
+    const float m = 1.0f + 2.5e-6f * P;
     // below q*: q = n / (2b + u)
     const float qa = n0 * cubic_rcp(fb + ua + 1e-30f);
-    const float qb = t1 > e1 ? n1 * cubic_rcp(fb + ub) : qs;
-    if (qa <= 1.00001f && qb >= -1.00001f)
-        cubic_one_band(A, qa, qb, fP, rho, kres, sh, B.k[0], B.n[0]);
+    const float qb = t1 > e ? n1 * cubic_rcp(fb + ub) : qs;
+    cubic_one_band(A, qa, qb, P, m + rho, m - rho, kres, sh, B.k[0], B.n[0]);
     // above q*: q = (2b + u) / (3a)
     if (qs <= 1.00001f)
-        cubic_one_band(A, (fb + ub) * A.r3a * 0.999996f, (fb + ua) * A.r3a * 1.000004f, fP, rho, kres,
-                       sh, B.k[1], B.n[1]);
+        cubic_one_band(A, (fb + ub) * A.r3a * 0.999996f, (fb + ua) * A.r3a * 1.000004f, P, m + rho,
+                       m - rho, kres, sh, B.k[1], B.n[1]);
+    return B;
 }
 
 // The candidate (from the job's d0 on) that the form (a, b, c, e0 - k) of a
 // band belongs to, or -1 when its discriminant is outside the window or the
 // form is not reduced.  Exact: P, Q, R are below 2^31 for a form in or next to
 // the window.
-EIS_HD int64_t cubic_hit(int kind, int32_t a, int32_t b, int32_t c, int32_t P, int32_t rho, int32_t e0,
-                         int32_t k, uint64_t d0, uint64_t ncand) {
-    const int32_t Q = rho + 9 * a * k;
-    const int32_t R = (int32_t)((uint32_t)c * (uint32_t)c - 3u * (uint32_t)b * (uint32_t)(e0 - k));
+EIS_HD int64_t cubic_hit(const CubicA &A, int32_t b, int32_t c, int32_t k, uint64_t d0, uint64_t ncand) {
+    const int kind = A.kind;
+    const int32_t a = A.a;
+    float cq, q2;
+    const int32_t rho = (int32_t)cubic_rho(A, (float)b, (float)c, cq, q2);
+    const int32_t e = b * ((int32_t)float_bits(cq) - 0x4B400000) + ((int32_t)float_bits(q2) - 0x4B400000) - k;
+    const int32_t P = b * b - 3 * a * c, Q = rho + 9 * a * k;
+    const int32_t R = (int32_t)((uint32_t)c * (uint32_t)c - 3u * (uint32_t)b * (uint32_t)e);
     if (Q > P || Q < -P || R < P) return -1;
     const int64_t D3 = 4 * (int64_t)P * R - (int64_t)Q * Q;  // 3 disc
     const int sh = kind ? 3 : 5;                             // 3 disc = 3d or 12d
@@ -302,11 +330,15 @@ inline void cubic_job_bounds(CubicJob &j) {
     j.amax = (uint32_t)(2.0 * r / std::sqrt(27.0) * (1 + 1e-9)) + 1;
     const uint32_t bmax = (uint32_t)(2.0 * r / std::sqrt(3.0) * (1 + 1e-9)) + 1;
     j.nblk = bmax / kCubicBlock + 1;
+    // about 0.41 (0.21) forms of kind 0 (1) a candidate, 0.6 of them at a = 1;
+    // slices of at least 8192 forms
+    const double forms = (j.kind ? 0.13 : 0.25) * (double)j.ncand / j.nblk;
+    j.slices = (uint32_t)std::fmin(64.0, std::fmax(1.0, forms / 8192.0));
 }
 
 // Units of a job.
 inline uint64_t cubic_units(const CubicJob &j) {
-    return (uint64_t)j.nblk * cubic_slices_below(j.amax + 1);
+    return (uint64_t)j.nblk * cubic_slices_below(j.amax + 1, j.slices);
 }
 
 }  // namespace eis

@@ -23,11 +23,10 @@ __device__ __forceinline__ int32_t warp_incl_scan(int32_t v, int lane) {
 }
 
 // Least lane whose inclusive prefix exceeds t (the owner of item t).
-template <int kLanes>
 __device__ __forceinline__ int scan_owner(int32_t incl, int32_t t) {
     int lo = 0;
 #pragma unroll
-    for (int s = kLanes / 2; s > 0; s >>= 1)
+    for (int s = 16; s > 0; s >>= 1)
         if (__shfl_sync(kFull, incl, lo + s - 1) <= t) lo += s;
     return lo;
 }
@@ -35,16 +34,17 @@ __device__ __forceinline__ int scan_owner(int32_t incl, int32_t t) {
 }  // namespace
 
 // One warp per unit (a; 16 consecutive b; a slice of the forms), units taken
-// from a global counter, small a first.  The warp finds the 16 ranges of c,
-// lays their (b, c) out flat, 32 at a time, one per lane; the lanes' bands of
-// forms are then laid out flat again and tested 32 at a time, so that lanes
-// stay busy whether a window holds thousands of forms per (b, c) or none.
-// Bound by instruction issue: 290 warp instructions for 32 (b, c), 83% of the
-// issue slots busy; the bitmaps stay in L2.  Measured: 0.55 ms for windows up
-// to 10^7 wide near 10^11, 1.9 ms near 10^12, about 11 ms near 2^44, and 1.0 ms
-// for the 10^9 window below 10^11, whose pass went from 827 to 45 ms (walk) and
-// from 425 to 38 ms (lane search) when the forms came in: 1.2e7 of its 1.0e8 d
-// are left, with a third of the period.
+// from a global counter, large b first (a unit has about 16 b / 3 values of c,
+// so that the last units are the short ones).  The warp finds the 16 ranges of
+// c and takes each 32 c at a time, one per lane; the lanes' bands of forms are
+// laid out flat and tested 32 at a time, so that lanes stay busy whether a
+// window holds thousands of forms per (b, c) or none.
+// Bound by instruction issue (150 warp instructions for 32 (b, c), 82% of the
+// issue slots busy); the bitmaps stay in L2.  Measured: 0.3 ms for windows up
+// to 10^7 wide near 10^11, 1.1 ms near 10^12, and 0.8 ms for the 10^9 window
+// below 10^11, whose pass went from 827 to 45 ms (walk) and from 425 to 38 ms
+// (lane search) when the forms came in: 1.2e7 of its 1.0e8 d are left, with a
+// third of the period.
 __global__ void __launch_bounds__(256) k_cubic(const CubicJob *__restrict__ jobs, uint32_t njobs,
                                                uint32_t nunits, uint32_t *__restrict__ next_ptr,
                                                uint32_t *__restrict__ bits0,
@@ -61,15 +61,16 @@ __global__ void __launch_bounds__(256) k_cubic(const CubicJob *__restrict__ jobs
             if (jobs[mid].unit0 <= u) jl = mid; else jh = mid;
         }
         const CubicJob job = jobs[jl];
-        const uint32_t v = u - job.unit0, blk = v % job.nblk;
-        uint32_t slice = v / job.nblk;
-        uint32_t a = 1;
-        while (a < 8 && slice >= cubic_slices(a)) slice -= cubic_slices(a++);
+        const uint32_t s1 = job.slices, v = u - job.unit0;
+        const uint32_t nsl = s1 == 1 ? job.amax : cubic_slices_below(job.amax + 1, s1);
+        const uint32_t blk = job.nblk - 1 - v / nsl;
+        uint32_t slice = v % nsl, a = s1 == 1 ? 8 : 1, nslices = 1;
+        while (a < 8 && slice >= (nslices = cubic_slices(a, s1))) slice -= cubic_slices(a++, s1);
         if (a == 8) {
-            a += slice;
+            a = (s1 == 1 ? 1 : 8) + slice;
             slice = 0;
+            nslices = 1;
         }
-        const uint32_t nslices = cubic_slices(a);
         const int kind = (int)job.kind;
         const CubicA A = cubic_a(job, (int32_t)a);
         const int32_t sh = cubic_shift(kind, A.a);
@@ -82,36 +83,32 @@ __global__ void __launch_bounds__(256) k_cubic(const CubicJob *__restrict__ jobs
         const float phi = __shfl_sync(kFull, pend, 2 * (lane & 15) + 1);
         int32_t c_first = 0, nc = 0;
         if (lane < 16 && cubic_pair_ok(kind, A.a, bm)) nc = cubic_c_range(A, bm, plo, phi, c_first);
-        const int32_t incl = warp_incl_scan(nc, lane);
-        const int32_t items = __shfl_sync(kFull, incl, 31);
-        for (int32_t base = 0; base < items; base += 32) {
-            const int32_t item = base + lane;
-            const int pair = scan_owner<16>(incl, min(item, items - 1));
-            const int32_t excl = __shfl_sync(kFull, incl - nc, pair);
-            const int32_t cf = __shfl_sync(kFull, c_first, pair);
-            const int32_t b = b0 + pair, c = cf + 2 * (item - excl);
-            CubicBands B;
-            B.n[0] = B.n[1] = 0;
-            if (item < items) cubic_bands(A, b, c, B);
-            const int32_t len = B.n[0] + B.n[1];
-            if (!__any_sync(kFull, len > 0)) continue;
-            const int32_t lin = warp_incl_scan(len, lane);
-            const int32_t total = __shfl_sync(kFull, lin, 31);
-            for (int32_t t0 = 32 * (int32_t)slice; t0 < total; t0 += 32 * (int32_t)nslices) {
-                const int32_t t = t0 + lane;
-                const int own = scan_owner<32>(lin, min(t, total - 1));
-                const int32_t i = t - __shfl_sync(kFull, lin - len, own);
-                const int32_t n0 = __shfl_sync(kFull, B.n[0], own);
-                const int32_t ka = __shfl_sync(kFull, B.k[0], own), kb = __shfl_sync(kFull, B.k[1], own);
-                const int32_t ob = __shfl_sync(kFull, b, own), oc = __shfl_sync(kFull, c, own);
-                const int32_t oP = __shfl_sync(kFull, B.P, own), orho = __shfl_sync(kFull, B.rho, own);
-                const int32_t oe = __shfl_sync(kFull, B.e0, own);
-                const int32_t k = i < n0 ? ka + (i << sh) : kb + ((i - n0) << sh);
-                if (t < total) {
-                    const int64_t h = cubic_hit(kind, A.a, ob, oc, oP, orho, oe, k, job.d0, job.ncand);
-                    if (h >= 0) {
-                        const uint64_t bit = job.bit0 + (uint64_t)h;
-                        atomicOr(&bits[bit >> 5], 1u << (bit & 31));
+        for (uint32_t pairs = __ballot_sync(kFull, nc > 0); pairs; pairs &= pairs - 1) {
+            const int pair = __ffs(pairs) - 1;
+            const int32_t b = b0 + pair, items = __shfl_sync(kFull, nc, pair);
+            const int32_t cf = __shfl_sync(kFull, c_first, pair) + 2 * lane;
+            for (int32_t base = 0; base < items; base += 32) {
+                const int32_t c = cf + 2 * base;
+                CubicBands B = cubic_bands(A, b, c);
+                if (base + lane >= items) B.n[0] = B.n[1] = 0;
+                const int32_t len = B.n[0] + B.n[1];
+                if (!__any_sync(kFull, len > 0)) continue;
+                const int32_t lin = warp_incl_scan(len, lane);
+                const int32_t total = __shfl_sync(kFull, lin, 31);
+                for (int32_t t0 = 32 * (int32_t)slice; t0 < total; t0 += 32 * (int32_t)nslices) {
+                    const int32_t t = t0 + lane;
+                    const int own = scan_owner(lin, min(t, total - 1));
+                    const int32_t i = t - __shfl_sync(kFull, lin - len, own);
+                    const int32_t n0 = __shfl_sync(kFull, B.n[0], own);
+                    const int32_t ka = __shfl_sync(kFull, B.k[0], own);
+                    const int32_t kb = __shfl_sync(kFull, B.k[1], own);
+                    const int32_t k = i < n0 ? ka + (i << sh) : kb + ((i - n0) << sh);
+                    if (t < total) {
+                        const int64_t h = cubic_hit(A, b, c + 2 * (own - lane), k, job.d0, job.ncand);
+                        if (h >= 0) {
+                            const uint64_t bit = job.bit0 + (uint64_t)h;
+                            atomicOr(&bits[bit >> 5], 1u << (bit & 31));
+                        }
                     }
                 }
             }

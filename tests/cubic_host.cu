@@ -30,14 +30,12 @@ int main() {
                 pairs += nc > 0;
                 for (int32_t i = 0; i < nc; ++i) {
                     const int32_t c = c0 + 2 * i;
-                    CubicBands B;
-                    cubic_bands(A, b, c, B);
+                    const CubicBands B = cubic_bands(A, b, c);
                     ++triples;
                     for (int w = 0; w < 2; ++w)
                         for (int32_t t = 0; t < B.n[w]; ++t) {
                             ++forms;
-                            const int64_t h = cubic_hit(kind, a, b, c, B.P, B.rho, B.e0, B.k[w] + st * t,
-                                                        d0, ncand);
+                            const int64_t h = cubic_hit(A, b, c, B.k[w] + st * t, d0, ncand);
                             if (h >= 0) bits[h] = '1';
                         }
                 }
