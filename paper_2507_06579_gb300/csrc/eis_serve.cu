@@ -253,7 +253,7 @@ bool launch_batch(eis_server *s, Slot &sl) {
                 ck(launch_k_bsgs(gb, st, fast, cv.giant_compose, sl.d_segs, nseg, sl.d_recs,
                                  sl.d_bctr + 1, C, sl.d_bctr + 3, sl.d_pool, sl.d_flags, nullptr,
                                  sl.d_steps + 1, sl.d_status, sl.d_fb, sl.d_bctr + 4, C, s->tt,
-                                 1u << 20, 1u << 14, 64));
+                                 1u << 20, 1u << 14, 64, dmax));
                 k_walk_persistent<<<s->grid, 256, 0, st>>>(sl.d_segs, nseg, sl.d_fb, sl.d_bctr + 4,
                                                            sl.d_bctr + 5, sl.d_flags, nullptr,
                                                            sl.d_steps, sl.d_status, s->step_limit, 0u,

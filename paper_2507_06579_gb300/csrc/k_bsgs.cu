@@ -358,9 +358,10 @@ __device__ __forceinline__ void bsgs_body(
     const unsigned char *__restrict__ pool, uint32_t *__restrict__ flags, uint8_t *__restrict__ glog,
     unsigned long long *__restrict__ acc, int *__restrict__ status, uint32_t *__restrict__ fb_list,
     uint32_t *__restrict__ fb_count, uint32_t fb_cap, const TuneTab &tt, uint32_t max_cycles,
-    uint32_t walk_cap, uint32_t walk_window, uint32_t *__restrict__ fp_all) {
+    uint32_t walk_cap, uint32_t walk_window, uint32_t walk_pause, uint32_t *__restrict__ fp_all) {
     const uint32_t n = min(*nrec, rec_cap);
     const uint32_t groups = (walk_window + kBsgsGroup - 1) / kBsgsGroup;
+    const uint32_t pause = min(groups, (walk_pause + kBsgsGroup - 1) / kBsgsGroup);
     const int lane = threadIdx.x & 31;
     const unsigned lt = lanemask_lt();
     uint32_t *fp_warp = fp_all + (threadIdx.x & ~31u) * kFpWords;  // lane t's words at t * kFpWords
@@ -498,7 +499,9 @@ __device__ __forceinline__ void bsgs_body(
         const bool went = walking;
         if (!walking) lean_park_idle(w, Cw);  // idle lanes step NaN states
         const uint32_t walked0 = walked;
-        for (uint32_t grp = 0; grp < groups && __any_sync(kFull, walking); ++grp) {
+        // (no limit once the records run out: then the longest search counts)
+        const uint32_t limit = exhausted ? groups : pause;
+        for (uint32_t grp = 0; grp < limit && __any_sync(kFull, walking); ++grp) {
 #pragma unroll
             for (int i = 0; i < kBsgsGroup; ++i) {
                 if (walking) {
@@ -593,11 +596,11 @@ __global__ void __launch_bounds__(128) k_bsgs_t(
     const unsigned char *__restrict__ pool, uint32_t *__restrict__ flags, uint8_t *__restrict__ glog,
     unsigned long long *__restrict__ acc, int *__restrict__ status, uint32_t *__restrict__ fb_list,
     uint32_t *__restrict__ fb_count, uint32_t fb_cap, const __grid_constant__ TuneTab tt,
-    uint32_t max_cycles, uint32_t walk_cap, uint32_t walk_window) {
+    uint32_t max_cycles, uint32_t walk_cap, uint32_t walk_window, uint32_t walk_pause) {
     __shared__ uint32_t fp_all[128 * kFpWords];
     bsgs_body<kFast, kCompose>(segs, nseg, recs, nrec, rec_cap, next_ptr, pool, flags, glog, acc,
                                status, fb_list, fb_count, fb_cap, tt, max_cycles, walk_cap,
-                               walk_window, fp_all);
+                               walk_window, walk_pause, fp_all);
 }
 
 // One instantiation per (quotient, composition), so that each kernel holds
@@ -616,14 +619,21 @@ cudaError_t launch_k_bsgs(uint32_t grid, cudaStream_t st, int fast, int compose,
                           uint32_t *next_ptr, const unsigned char *pool, uint32_t *flags,
                           uint8_t *glog, unsigned long long *acc, int *status, uint32_t *fb_list,
                           uint32_t *fb_count, uint32_t fb_cap, const TuneTab &tt,
-                          uint32_t max_cycles, uint32_t walk_cap, uint32_t walk_window) {
+                          uint32_t max_cycles, uint32_t walk_cap, uint32_t walk_window,
+                          uint64_t d_max) {
     TuneTab t = tt;
+    // A warp's walks pause after 4/3 of their mean length m: at m = 12 / 16 / 24
+    // the search of the window's 1.2e7 d takes 11.5 / 11.7 / 12.8 ms pausing after
+    // 16 steps, 11.8 / 11.7 / 12.2 after 32, 12.4 / 12.7 / 13.3 after 64.  (A
+    // window above 2^12 asks for walks that are not cut.)
+    const float m = 1.39f / tt.tau[tune_row(tt, d_max)];
+    uint32_t walk_pause = walk_window > 4096 ? walk_window : std::max(16u, (uint32_t)(1.34f * m));
     k_prep<<<std::min(rec_cap / 128 + 1, 4 * grid), 128, 0, st>>>(
         segs, nseg, const_cast<DRecord *>(recs), nrec, rec_cap, pool, tt);
     if (cudaError_t e = cudaPeekAtLastError(); e != cudaSuccess) return e;
     void *args[] = {&segs, &nseg, &recs, &nrec, &rec_cap, &next_ptr, &pool, &flags, &glog,
                     &acc, &status, &fb_list, &fb_count, &fb_cap, &t, &max_cycles, &walk_cap,
-                    &walk_window};
+                    &walk_window, &walk_pause};
     return cudaLaunchKernel(k_bsgs_kernel(fast, compose), dim3(grid), dim3(128), args, 0, st);
 }
 
