@@ -47,6 +47,7 @@ struct eis_ctx {
     uint64_t *d_sqtab = nullptr;  // per odd prime p: (p^2)^(-1) mod 2^64, floor((2^64-1)/p^2)
     uint32_t nprimes = 0;
     std::vector<uint32_t> primes;  // host copy of the odd primes of d_primes
+    uint32_t np_small = 0;         // of which below kSieveSplit
     int *d_single = nullptr;  // [0] result, [1] steps, [2] status
     unsigned char *d_query = nullptr;  // K3 single query: u64 d, i8 out, int status, u64 acc[2], u32 next
     QueryOut *h_query = nullptr;       // k_query's answer: pinned host memory the device writes
@@ -272,6 +273,16 @@ static std::vector<uint32_t> odd_primes_below(uint32_t n) {
     return out;
 }
 
+// Number of odd primes p of the table with p^2 <= d.
+static uint32_t primes_up_to(const eis_ctx *c, uint64_t d) {
+    uint64_t r = (uint64_t)std::sqrt((double)d);
+    while (r * r > d) --r;
+    while ((r + 1) * (r + 1) <= d) ++r;
+    return (uint32_t)(std::upper_bound(c->primes.begin(), c->primes.end(),
+                                       (uint32_t)std::min<uint64_t>(r, UINT32_MAX)) -
+                      c->primes.begin());
+}
+
 // Bytes a plan needs per candidate: survivor queue (4) + two bitmaps (1/4),
 // plus the optional per-candidate log byte.
 static uint64_t max_chunk_cands(eis_ctx *c, int with_log) {
@@ -400,9 +411,10 @@ static int plan_enqueue(eis_plan *p, cudaStream_t s, bool capturing) {
     EIS_CK(cudaMemsetAsync(p->d_res, 0, p->res_bytes, s));
     if (p->d_glog) EIS_CK(cudaMemsetAsync(p->d_glog, 0, p->total_cand, s));
     if (ntiles > 0) {
-        k_sieve<<<ntiles, 256, 0, s>>>(p->d_tiles, p->d_segs, c->d_primes, c->nprimes, p->d_sqfree,
-                                       p->d_tile_pop, p->primes_only);
-        ++launches;
+        const int sieves = launch_sieve(ntiles, s, p->d_tiles, p->d_segs, nseg, c->d_primes, c->d_sqtab,
+                                        c->nprimes, c->np_small, primes_up_to(c, p->d_max),
+                                        p->d_sqfree, p->d_tile_pop, p->primes_only);
+        launches += sieves;
         if (p->mode == EIS_MODE_PERSISTENT) {
             const bool cubic = !p->cubic.empty();
             if (cubic) {
@@ -413,6 +425,10 @@ static int plan_enqueue(eis_plan *p, cudaStream_t s, bool capturing) {
                 k_select<<<ntiles, 256, 0, s>>>(p->d_tiles, p->d_sqfree, p->d_flags, p->d_field,
                                                 p->d_segfield, p->d_glog, p->d_tile_pop);
                 launches += 2;
+            } else if (sieves > 1) {
+                k_select<<<ntiles, 256, 0, s>>>(p->d_tiles, p->d_sqfree, nullptr, nullptr, nullptr,
+                                                nullptr, p->d_tile_pop);
+                ++launches;
             }
             k_scan_tiles<<<1, 1024, 0, s>>>(p->d_tile_pop, p->d_tile_off, ntiles, p->d_ctr);
             k_compact<<<ntiles, 256, 0, s>>>(p->d_tiles, p->d_sqfree, p->d_tile_off, p->d_surv,
@@ -951,11 +967,14 @@ eis_ctx_view eis_ctx_get_view(eis_ctx *c) {
     v.giant_grid = (uint32_t)(c->sm_count * 4);
     v.giant_compose = c->giant_compose;
     v.step_limit = (uint32_t)std::min<int64_t>(c->step_limit, 0xffffffffll);
+    v.np_small = c->np_small;
     v.sm_count = (uint32_t)c->sm_count;
     v.bsgs_grid = (uint32_t)(c->sm_count * c->occ_bsgs);
     v.own_settings = c->step_limit >= kCubicMinStepLimit;
     return v;
 }
+
+uint32_t eis_ctx_primes_up_to(eis_ctx *c, uint64_t d) { return primes_up_to(c, d); }
 
 void eis_ctx_search_rows(eis_ctx *c, TuneTab &tt) {
     if (c->tune.empty())
@@ -1037,6 +1056,7 @@ int eis_create(eis_ctx **out, int device, uint64_t mem_budget_bytes) {
     std::vector<uint32_t> pr = odd_primes_below(1u << 22);
     c->nprimes = (uint32_t)pr.size();
     c->primes = pr;
+    c->np_small = (uint32_t)(std::lower_bound(pr.begin(), pr.end(), kSieveSplit) - pr.begin());
     // Every table of the context is charged once: primes, the square-free
     // test table (16 B per prime), the single-query words.
     if (!ctx_reserve(c, pr.size() * 4 + pr.size() * 16 + 4 * sizeof(int) + 64)) {
@@ -1628,12 +1648,7 @@ int eis_is_eisenstein(eis_ctx *c, uint64_t d, int *result_out) {
     int res = 0;  // 0: not in D, else 1 + log eps_d
     // only odd primes with p^2 <= d can divide d: scan those, on as many
     // blocks as they fill (at most two per SM)
-    uint64_t r = (uint64_t)std::sqrt((double)d);
-    while (r * r > d) --r;
-    while ((r + 1) * (r + 1) <= d) ++r;
-    const uint32_t np = (uint32_t)(std::upper_bound(c->primes.begin(), c->primes.end(),
-                                                    (uint32_t)std::min<uint64_t>(r, UINT32_MAX)) -
-                                   c->primes.begin());
+    const uint32_t np = primes_up_to(c, d);
     const uint32_t blocks = std::max<uint32_t>(1u, std::min<uint32_t>((np + 255) / 256,
                                                                       (uint32_t)c->sm_count * 2));
     if (c->mode == EIS_MODE_PERSISTENT && c->giant_compose == EIS_COMPOSE_TEXTBOOK) {

@@ -49,6 +49,7 @@ namespace eis {
 constexpr int kTileCands = 1 << 16;          // candidates per sieve tile
 constexpr int kTileWords = kTileCands / 32;  // bitmap words per tile
 constexpr int kPlainBlockCands = 1 << 21;    // 2^24-wide block of d = 2^21 candidates
+constexpr uint32_t kSieveSplit = 512;        // primes from here on: k_sieve_big
 constexpr float kMagic = 8388608.0f;         // 2^23
 constexpr unsigned kFull = 0xffffffffu;
 

@@ -56,7 +56,7 @@
 
 namespace eis {
 
-constexpr int kCubicBlock = 16;  // values of b a unit of work holds
+constexpr int kCubicBlock = 8;  // values of b a unit of work holds (at most 16)
 
 // One enumeration: the forms of kind `kind` whose d lies among the ncand
 // candidates from d0 on.
@@ -72,7 +72,7 @@ struct CubicJob {
     uint32_t pad;
 };
 
-// Slices a unit (a; 16 b's) is cut into, of s1 at a = 1: the forms of a window
+// Slices a unit (a; 8 b's) is cut into, of s1 at a = 1: the forms of a window
 // thin out like 1/a^2, and a slice takes every S-th of 32 forms (but looks at
 // every c, so that narrow windows have s1 = 1).
 EIS_HD uint32_t cubic_slices(uint32_t a, uint32_t s1) { return a * a < s1 ? s1 / (a * a) : 1u; }

@@ -16,7 +16,7 @@ struct eis_ctx_view {
     int device;
     const uint32_t *d_primes;  // odd primes < 2^22 on the device
     const uint64_t *d_sqtab;   // their division-free square-divisibility table
-    uint32_t nprimes;
+    uint32_t nprimes, np_small;  // all, and those below kSieveSplit
     uint32_t walk_grid;        // persistent walk grid (SMs x resident CTAs)
     uint32_t giant_grid;       // one-warp blocks of k_giant that fit at once (SMs x 4)
     int giant_compose;         // EIS_COMPOSE_*
@@ -36,6 +36,8 @@ void eis_ctx_search_rows(eis_ctx *ctx, eis::TuneTab &tt);
 void eis_giant_params(uint64_t d, int64_t forced, int &nbaby, int &log2n);
 
 eis_ctx_view eis_ctx_get_view(eis_ctx *ctx);
+// Odd primes p of the table with p^2 <= d.
+uint32_t eis_ctx_primes_up_to(eis_ctx *ctx, uint64_t d);
 // Account `bytes` of device memory against the context budget; false if over.
 bool eis_ctx_reserve(eis_ctx *ctx, uint64_t bytes);
 void eis_ctx_release(eis_ctx *ctx, uint64_t bytes);

@@ -12,6 +12,14 @@ namespace eis {
 
 __global__ void k_sieve(const Tile *tiles, const Seg *segs, const uint32_t *primes,
                         uint32_t nprimes, uint32_t *sqfree, uint32_t *tile_pop, int primes_only);
+__global__ void k_sieve_big(const Seg *segs, uint32_t nseg, const uint32_t *primes,
+                            const uint64_t *sqtab, uint32_t nprimes, uint32_t *sqfree);
+// k_sieve, with k_sieve_big where it pays; np primes have p^2 <= the largest d,
+// nsmall of the table are below kSieveSplit.  Returns the kernels launched (2: tile_pop
+// does not count what k_sieve_big cleared).
+int launch_sieve(uint32_t ntiles, cudaStream_t st, const Tile *tiles, const Seg *segs, uint32_t nseg,
+                 const uint32_t *primes, const uint64_t *sqtab, uint32_t nprimes, uint32_t nsmall,
+                 uint32_t np, uint32_t *sqfree, uint32_t *tile_pop, int primes_only);
 __global__ void k_scan_tiles(const uint32_t *tile_pop, uint32_t *tile_off, uint32_t ntiles,
                              uint32_t *total);
 __global__ void k_compact(const Tile *tiles, const uint32_t *sqfree, const uint32_t *tile_off,

@@ -229,8 +229,11 @@ bool launch_batch(eis_server *s, Slot &sl) {
     uint64_t dmax = 0;
     for (const Part &p : sl.items) dmax = std::max(dmax, p.d0 + 8 * (p.ncand - 1));
     if (nt > 0) {
-        k_sieve<<<nt, 256, 0, st>>>(sl.d_tiles, sl.d_segs, cv.d_primes, cv.nprimes, sl.d_sqfree,
-                                    sl.d_tile_pop, 0);
+        if (launch_sieve(nt, st, sl.d_tiles, sl.d_segs, nseg, cv.d_primes, cv.d_sqtab, cv.nprimes,
+                         cv.np_small, eis_ctx_primes_up_to(s->ctx, dmax), sl.d_sqfree, sl.d_tile_pop,
+                         0) > 1)
+            k_select<<<nt, 256, 0, st>>>(sl.d_tiles, sl.d_sqfree, nullptr, nullptr, nullptr, nullptr,
+                                         sl.d_tile_pop);
         k_scan_tiles<<<1, 1024, 0, st>>>(sl.d_tile_pop, sl.d_tile_off, nt, sl.d_ctr);
         k_compact<<<nt, 256, 0, st>>>(sl.d_tiles, sl.d_sqfree, sl.d_tile_off, sl.d_surv, nullptr,
                                       nullptr, nullptr);

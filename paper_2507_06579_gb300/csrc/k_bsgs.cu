@@ -590,7 +590,7 @@ __device__ __forceinline__ void bsgs_body(
 }  // namespace
 
 template <bool kFast, int kCompose>
-__global__ void __launch_bounds__(128) k_bsgs_t(
+__global__ void __launch_bounds__(128, kCompose == 0 ? 8 : 1) k_bsgs_t(
     const Seg *__restrict__ segs, uint32_t nseg, const DRecord *__restrict__ recs,
     const uint32_t *__restrict__ nrec, uint32_t rec_cap, uint32_t *__restrict__ next_ptr,
     const unsigned char *__restrict__ pool, uint32_t *__restrict__ flags, uint8_t *__restrict__ glog,

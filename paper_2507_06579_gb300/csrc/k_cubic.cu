@@ -33,9 +33,9 @@ __device__ __forceinline__ int scan_owner(int32_t incl, int32_t t) {
 
 }  // namespace
 
-// One warp per unit (a; 16 consecutive b; a slice of the forms), units taken
-// from a global counter, large b first (a unit has about 16 b / 3 values of c,
-// so that the last units are the short ones).  The warp finds the 16 ranges of
+// One warp per unit (a; 8 consecutive b; a slice of the forms), units taken
+// from a global counter, large b first (a unit has about 8 b / 3 values of c,
+// so that the last units are the short ones).  The warp finds the 8 ranges of
 // c and takes each 32 c at a time, one per lane; the lanes' bands of forms are
 // laid out flat and tested 32 at a time, so that lanes stay busy whether a
 // window holds thousands of forms per (b, c) or none.
@@ -82,7 +82,7 @@ __global__ void __launch_bounds__(256) k_cubic(const CubicJob *__restrict__ jobs
         const float plo = __shfl_sync(kFull, pend, 2 * (lane & 15));
         const float phi = __shfl_sync(kFull, pend, 2 * (lane & 15) + 1);
         int32_t c_first = 0, nc = 0;
-        if (lane < 16 && cubic_pair_ok(kind, A.a, bm)) nc = cubic_c_range(A, bm, plo, phi, c_first);
+        if (lane < kCubicBlock && cubic_pair_ok(kind, A.a, bm)) nc = cubic_c_range(A, bm, plo, phi, c_first);
         for (uint32_t pairs = __ballot_sync(kFull, nc > 0); pairs; pairs &= pairs - 1) {
             const int pair = __ffs(pairs) - 1;
             const int32_t b = b0 + pair, items = __shfl_sync(kFull, nc, pair);
@@ -117,8 +117,8 @@ __global__ void __launch_bounds__(256) k_cubic(const CubicJob *__restrict__ jobs
 }
 
 // After the sieve and k_cubic: flags &= square-free, and per tile the number
-// of candidates left to the walk (`left_word`).  glog (or null): 1 where the
-// flag is set.
+// of candidates left to the walk (`left_word`).  flags null: only the count.
+// glog (or null): 1 where the flag is set.
 __global__ void __launch_bounds__(256) k_select(const Tile *__restrict__ tiles,
                                                 const uint32_t *__restrict__ sqfree,
                                                 uint32_t *__restrict__ flags,
@@ -133,8 +133,8 @@ __global__ void __launch_bounds__(256) k_select(const Tile *__restrict__ tiles,
     const bool use = field && seg_field[t.seg];
     uint32_t pop = 0;
     for (uint32_t w = threadIdx.x; w < nw; w += blockDim.x) {
-        const uint32_t sq = sqfree[wbase + w], f = flags[wbase + w] & sq;
-        flags[wbase + w] = f;
+        const uint32_t sq = sqfree[wbase + w], f = flags ? flags[wbase + w] & sq : 0u;
+        if (flags) flags[wbase + w] = f;
         pop += __popc(left_word(sq, f, use ? field[wbase + w] : kFull));
         if (glog)
             for (uint32_t x = f; x; x &= x - 1) glog[32 * (wbase + w) + (__ffs(x) - 1)] = 1;

@@ -114,6 +114,36 @@ __global__ void __launch_bounds__(256) k_sieve(const Tile *__restrict__ tiles,
     if (threadIdx.x == 0) tile_pop[blockIdx.x] = pop;
 }
 
+// The larger primes, one thread per prime and interval: primes[0 .. nprimes)
+// with their squares' inverses (sqtab[2i + 1] = floor((2^64 - 1) / p^2)).  Their
+// hits in an interval of n candidates are n / p^2, so that taking them tile by
+// tile in k_sieve spent nearly all its divisions on primes without a hit in
+// the tile, and a plan of a few tiles ran on as many SMs: 2.5e5 candidates
+// below 2^44 (295,000 primes, 4 tiles) 883 -> 21 us with k_sieve, 1.2e6 near
+// 10^11 86 -> 19.
+// The quotient is one high product, off by at most one.
+__global__ void __launch_bounds__(256) k_sieve_big(const Seg *__restrict__ segs, uint32_t nseg,
+                                                   const uint32_t *__restrict__ primes,
+                                                   const uint64_t *__restrict__ sqtab,
+                                                   uint32_t nprimes, uint32_t *__restrict__ sqfree) {
+    const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= nprimes) return;
+    const uint64_t p2 = (uint64_t)primes[i] * primes[i], lim = sqtab[2 * i + 1];
+    for (uint32_t si = blockIdx.y; si < nseg; si += gridDim.y) {
+        const Seg s = segs[si];
+        if (s.ncand == 0) continue;
+        const uint64_t dlast = s.d0 + 8 * (s.ncand - 1);
+        if (p2 > dlast) continue;
+        uint64_t m = __umul64hi(s.d0, lim);  // floor(d0 / p^2) or one less
+        while (m * p2 < s.d0) ++m;
+        m += (13 - m % 8) % 8;  // m == 5 (mod 8)
+        for (uint64_t dh = m * p2; dh <= dlast; dh += 8 * p2) {
+            const uint64_t bit = s.cand0 + ((dh - s.d0) >> 3);
+            atomicAnd(&sqfree[bit >> 5], ~(1u << (bit & 31)));
+        }
+    }
+}
+
 // Exclusive scan of tile_pop into tile_off (single CTA) and the total.
 __global__ void __launch_bounds__(1024) k_scan_tiles(const uint32_t *__restrict__ tile_pop,
                                                      uint32_t *__restrict__ tile_off,
@@ -230,6 +260,22 @@ __global__ void k_fill(uint32_t *__restrict__ buf, uint64_t nwords, uint32_t v) 
     for (uint64_t k = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; k < nwords;
          k += (uint64_t)gridDim.x * blockDim.x)
         buf[k] = v;
+}
+
+// Up to 4096 the tile's own pass over the primes is short.
+int launch_sieve(uint32_t ntiles, cudaStream_t st, const Tile *tiles, const Seg *segs, uint32_t nseg,
+                 const uint32_t *primes, const uint64_t *sqtab, uint32_t nprimes, uint32_t nsmall,
+                 uint32_t np, uint32_t *sqfree, uint32_t *tile_pop, int primes_only) {
+    const bool big = !primes_only && np > nsmall + 512;
+    k_sieve<<<ntiles, 256, 0, st>>>(tiles, segs, primes, big ? nsmall : nprimes, sqfree, tile_pop,
+                                    primes_only);
+    if (!big) return 1;
+    const uint32_t n = np - nsmall;
+    // a thread takes several intervals with its prime when there are many
+    const uint32_t gx = (n + 255) / 256, gy = 2432 / gx + 1;
+    k_sieve_big<<<dim3(gx, nseg < gy ? nseg : gy), 256, 0, st>>>(
+        segs, nseg, primes + nsmall, sqtab + 2 * nsmall, n, sqfree);
+    return 2;
 }
 
 }  // namespace eis
