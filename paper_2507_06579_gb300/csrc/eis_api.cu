@@ -296,6 +296,20 @@ static uint64_t max_chunk_cands(eis_ctx *c, int with_log) {
     return m;
 }
 
+// Candidates per tile of a plan: halved from 2^16, not below 2^13, while the
+// tiles are fewer than two per SM.  The tile kernels are one block a tile and
+// short serial loops over it: 1.25e6 candidates, 20 tiles -> 153, k_select
+// 18.4 -> 5.5 us, k_compact 22.3 -> 5.6.  With two blocks an SM in flight shorter
+// tiles only repeat the work a tile takes whatever its length.  Tables of more
+// tiles are taken only with twice the plan's room left.
+static uint32_t tile_cands(eis_ctx *c, uint64_t ncand) {
+    uint32_t t = kTileCands;
+    const uint64_t used = c->in_use.load();
+    if (c->budget < used || c->budget - used < (1u << 20) + 16 * ncand) return t;
+    while (t > kTileCands / 8 && ncand < 2 * (uint64_t)c->sm_count * t) t /= 2;
+    return t;
+}
+
 // Baby-step count N of the giant-step search for discriminants up to d: about
 // twice the square root of a typical period (~0.13 sqrt(d) steps), a power of
 // two in [256, 4096]; the table holds 4N entries (load <= 1/2).
@@ -573,10 +587,11 @@ static int plan_build(eis_ctx *c, const uint64_t *lo, const uint64_t *hi, size_t
         plan_free(p);
         return EIS_ENOMEM;
     }
+    const uint32_t tile = tile_cands(c, cur);
     for (uint32_t si = 0; si < p->segs.size(); ++si) {
         const Seg &s = p->segs[si];
-        for (uint64_t off = 0; off < s.ncand; off += kTileCands) {
-            Tile t{s.cand0 + off, si, (uint32_t)std::min<uint64_t>(kTileCands, s.ncand - off)};
+        for (uint64_t off = 0; off < s.ncand; off += tile) {
+            Tile t{s.cand0 + off, si, (uint32_t)std::min<uint64_t>(tile, s.ncand - off)};
             p->tiles.push_back(t);
         }
         for (uint64_t off = 0; off < s.ncand; off += kPlainBlockCands) {

@@ -40,3 +40,23 @@ def test_square_free_bitmap(lo, n):
             bits = np.unpackbits(sq[off:].view(np.uint8), bitorder="little")[:len(ref)]
             p.destroy()
             assert np.array_equal(bits, ref)
+
+
+@pytest.mark.parametrize("lo,n", [(5, 8_191), (10**9, 8_193), (10**10, 98_304), (10**9, 1_245_185)])
+def test_short_tiles(lo, n):
+    """A small plan's shorter tiles give what whole ones give (a context
+    without room for the longer tile table), classes and counts included."""
+    E.build()
+    got = []
+    with E.Context(0) as ctx:
+        used0 = ctx.get_option(E.EIS_OPT_MEM_IN_USE)
+    for budget in (0, used0 + (1 << 20) + 12 * n):
+        with E.Context(0, budget) as ctx:
+            p = ctx.plan_create([lo, lo + 8 * n + 64], [lo + 8 * n, lo + 8 * n + 800],
+                                E.EIS_MODE_PERSISTENT, E.EIS_PLAN_CLASSES)
+            p.launch()
+            flags, sq = p.copy_bitmaps()
+            got.append((flags.tobytes(), sq.tobytes(), p.counts().tolist(), p.counts_D().tolist(),
+                        p.class_counts().tolist()))
+            p.destroy()
+    assert got[0] == got[1]
