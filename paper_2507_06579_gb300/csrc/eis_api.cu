@@ -362,8 +362,18 @@ static constexpr double kCubicMinGain = 4e8;
 // periods are a third, 512 / 768..1024 / 1536 / 2048..3072 (coef 1.62).  Below
 // 5e8 (2e9 for what the forms leave) walking to the centre is as fast: 2.06
 // against 2.63 ms for 2e8 d's width at 10^9, 3.5 against 2.9 for all d.
-static void auto_rows(TuneTab &tt, bool after_forms) {
-    const double coef = after_forms ? 1.62 : 2.43;
+//
+// A plan of few d ends with its longest searches, each on one lane, so longer
+// walks and denser tables (80 marks) pay: with left d's and lanes that search,
+// N grows by (4 lanes / left)^0.3, up to 2.8 (lanes = 0: not at all).  Best factor
+// of 1 / 1.4 / 2 / 2.8 / 4 measured: 2.8 for 9,700 d near 10^12 (1.40 -> 0.98 ms), 2.8 for
+// 30,000 below 2^44 (4.16 -> 3.48), 2 for 97,000 near 10^12 (1.98 -> 1.48), 1.4
+// for 124,000 near 10^11 (0.948 -> 0.913 a call) and 200,000 below 2^44 (7.0 ->
+// 6.77).  A server's rounds of 2^18 from four slots take none (factors above 2:
+// +2 to +7%).
+static void auto_rows(TuneTab &tt, bool after_forms, uint64_t left, uint64_t lanes) {
+    const double few = std::min(2.8, std::pow(4.0 * (double)lanes / (double)(left + 1), 0.3));
+    const double coef = (after_forms ? 1.62 : 2.43) * std::max(1.0, few);
     double hi = after_forms ? 2e9 : 5e8;
     const double step = after_forms ? 4.0 : 5.0;
     tt.n = kTuneRows;
@@ -371,7 +381,7 @@ static void auto_rows(TuneTab &tt, bool after_forms) {
         tt.d_hi[r] = r + 1 < kTuneRows ? (uint64_t)hi : EIS_D_LIMIT;
         const double N = coef * std::sqrt(std::sqrt(0.5 * hi));
         tt.nbaby[r] = r == 0 ? 0u : (uint32_t)(N / 64.0 + 0.5) * 64u;
-        const double m = std::min(64.0, std::max(12.0, N / 56.0));
+        const double m = few > 1.0 ? std::max(12.0, N / 80.0) : std::min(64.0, std::max(12.0, N / 56.0));
         tt.tau[r] = (float)(1.39 / m);
     }
 }
@@ -631,7 +641,7 @@ static int plan_build(eis_ctx *c, const uint64_t *lo, const uint64_t *hi, size_t
     bool any_search = false;
     const bool own = c->tune.empty() && c->giant_threshold == 0 && c->step_limit >= kCubicMinStepLimit;
     if (own) {
-        auto_rows(p->tt, false);
+        auto_rows(p->tt, false, 0, 0);
         for (const Seg &sg : p->segs)
             any_search |= sg.ncand && sg.d0 + 8 * (sg.ncand - 1) >= p->tt.d_hi[0];
     } else if (!c->tune.empty()) {
@@ -687,8 +697,8 @@ static int plan_build(eis_ctx *c, const uint64_t *lo, const uint64_t *hi, size_t
         left += plain ? p->segs[si].ncand : p->segs[si].ncand * 15 / 100 + 64;
         left_walk += plain ? p->segs[si].ncand : 0;
     }
-    if (own && left_walk < left / 2) {
-        auto_rows(p->tt, true);
+    if (own) {
+        auto_rows(p->tt, left_walk < left / 2, left, (uint64_t)c->sm_count * c->occ_bsgs * 128);
         any_search = false;
         for (const Seg &sg : p->segs)
             any_search |= sg.ncand && sg.d0 + 8 * (sg.ncand - 1) >= p->tt.d_hi[0];
@@ -993,7 +1003,7 @@ uint32_t eis_ctx_primes_up_to(eis_ctx *c, uint64_t d) { return primes_up_to(c, d
 
 void eis_ctx_search_rows(eis_ctx *c, TuneTab &tt) {
     if (c->tune.empty())
-        auto_rows(tt, false);
+        auto_rows(tt, false, 0, 0);
     else
         tune_rows(c, tt);
 }
