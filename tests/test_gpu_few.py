@@ -21,12 +21,12 @@ def test_few_d_equal_the_walk(lo, n):
     for limit in (1 << 26, 1 << 25):  # own settings; every d walked
         with E.Context(0) as ctx:
             ctx.set_option(E.EIS_OPT_STEP_LIMIT, limit)
-            p = ctx.plan_create([lo], [hi], E.EIS_MODE_PERSISTENT)
+            p = ctx.plan_create([lo], [hi], E.EIS_MODE_PERSISTENT, E.EIS_PLAN_CLASSES)
             p.launch()
             flags, sq = p.copy_bitmaps()
             deferred = p.stats()["deferred"]
             p.destroy()
-            got.append((flags.tobytes(), sq.tobytes(),
+            got.append((flags.tobytes(), sq.tobytes(), ctx.class_counts(lo, hi),
                         ctx.classify_range_log(lo, hi).tobytes()))
         assert (deferred > 0) == (limit == 1 << 26)
     assert got[0] == got[1]
