@@ -63,9 +63,18 @@ extern "C" {
 /* Execution modes (eis_set_option(EIS_OPT_MODE)). */
 #define EIS_MODE_PLAIN 0      /* one launch per 2^24-wide block of d, one    */
                               /* thread per candidate                         */
-#define EIS_MODE_PERSISTENT 1 /* sieve + compaction + one persistent launch   */
-                              /* whose lanes steal d's from a global queue   */
+#define EIS_MODE_PERSISTENT 1 /* sieve; cubic forms where they pay (see below) */
+                              /* decide most d; the rest go through a queue   */
+                              /* that resident lanes steal d's from           */
                               /* (CUDA-graph captured per plan)               */
+
+/* Cubic forms: d is in E when a cubic field of discriminant 4d exists, and not
+ * in E when there is none of discriminant 4d or d (class field theory), so an
+ * enumeration of reduced binary cubic forms over an interval decides most of
+ * its d without their units.  Plans use it, per interval, where it costs less
+ * than the walks it saves, while EIS_OPT_STEP_LIMIT is at its default or above;
+ * a lower limit asks that every d be walked and held to it.  The results are
+ * the same; baby_steps and giant_steps count the d that were walked. */
 
 /* Options (eis_set_option / eis_get_option). */
 #define EIS_OPT_MODE 1           /* EIS_MODE_*; default EIS_MODE_PERSISTENT   */
@@ -97,8 +106,9 @@ extern "C" {
                                  /* without meeting a marked state before its  */
                                  /* d is finished by the plain walk (2^14)     */
 #define EIS_OPT_BSGS_WINDOW 15   /* lane search: steps a lane walks per search */
-                                 /* iteration before the warp's composition    */
-                                 /* (64; 0: until every lane's walk has ended) */
+                                 /* iteration before the warp's composition, at */
+                                 /* most (64; 0: until every lane's walk has    */
+                                 /* ended); a warp may pause sooner             */
 
 /* Giant-step searches of plans (EIS_OPT_GIANT_KERNEL).  Both run after
  * EIS_OPT_GIANT_THRESHOLD baby steps without a centre. */
@@ -202,11 +212,11 @@ int eis_classify_range_log(eis_ctx *ctx, uint64_t lo, uint64_t hi, uint8_t *log_
  * d not in D (d != 5 mod 8, or p^2 | d for an odd prime p): EIS_ENOTD and
  * nothing written; d >= EIS_D_LIMIT: EIS_ERANGE; a walk or giant-step
  * search past its limit: EIS_ESTEPS.  The square-free test spreads the prime
- * table over the whole GPU; then, in EIS_MODE_PERSISTENT (default), one warp
- * runs the baby-step giant-step search of Algorithm 1 (composition per
- * EIS_OPT_GIANT_COMPOSE), and in EIS_MODE_PLAIN one lane walks the half
- * period.  Synchronous on the context's stream; eis_get_stats reports the
- * baby and giant steps taken. */
+ * table over the whole GPU.  In EIS_MODE_PERSISTENT (default) one block runs
+ * the baby-step giant-step search of Algorithm 1 in the same launch (with
+ * EIS_COMPOSE_NUCOMP, one warp after it), and in EIS_MODE_PLAIN one lane walks
+ * the half period.  Synchronous on the context's stream; eis_get_stats reports
+ * the baby and giant steps taken. */
 int eis_is_eisenstein(eis_ctx *ctx, uint64_t d, int *result_out);
 
 /* counts_out[i] = #E cap [lo[i], hi[i]) for i < n, all intervals classified

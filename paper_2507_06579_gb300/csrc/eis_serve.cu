@@ -99,7 +99,7 @@ struct eis_server {
     // The lane search (eis_bsgs.cuh) takes the walks instead, in rounds of
     // search_chunk survivors, when the server runs at its default giant_after
     // and the slots' tables fit an eighth of the budget: 2000 requests of the
-    // serving mix at once take 48 ms against 134 (walks, and the longest handed
+    // serving mix at once take 44 ms against 133 (walks, and the longest handed
     // to the warp-per-d kernel).
     uint32_t search_chunk = 0;  // 0: walk
     uint32_t rec_grid = 0, bsgs_grid = 0;
