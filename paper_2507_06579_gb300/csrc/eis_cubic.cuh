@@ -169,7 +169,8 @@ EIS_HD int32_t cubic_floordiv(int32_t x, int32_t m, float rm, int32_t &rem) {
 struct CubicA {
     int32_t a, kind;
     float K0h, K0l;   // 9a disc at the window's least end, in two floats
-    float dK;         // ... and what it grows by to the other
+    float dK;         // ... and what it grows by to the other, and by 10^-6 more: past the
+                      // error of dK / P^2 (2^-22), whole candidates of a wide window
     float k0, k1;     // 27 a^2 disc / 4 there
     float pmax;       // sqrt of the largest discriminant, widened
     float r9a, r3a;   // 1/(9a), 1/(3a)
@@ -184,7 +185,7 @@ EIS_HD CubicA cubic_a(const CubicJob &j, int32_t a) {
     const int64_t K0 = 9 * a * D0, K1 = 9 * a * D1;  // < 9 * 1115 * 2^46
     A.K0h = (float)K0;
     A.K0l = (float)(K0 - (int64_t)A.K0h);
-    A.dK = (float)(K1 - K0);
+    A.dK = (float)(K1 - K0) * 1.000001f;
     const float s = 0.75f * (float)a;
     A.k0 = s * A.K0h;
     A.k1 = s * (float)K1;
@@ -285,16 +286,20 @@ EIS_HD CubicBands cubic_bands(const CubicA &A, int32_t b, int32_t c) {
     const float n0 = cubic_fma(4.0f, fc, z) + zc, n1 = cubic_fma(A.dK, rp, n0);
     const float fb = 2.0f * fb1, fb2 = fb * fb;
     const float t0 = cubic_fma(-fa, n0, fb2), t1 = cubic_fma(-fa, n1, fb2);
-    // 1e-6 (4b^2 + 3a |n|) at the larger of the two
-    const float e = 1e-6f * (2.0f * fb2 + fmaxf(fabsf(t0), fabsf(t1)));
-    if (t0 + e < 0.0f) return B;  // the window lies above the largest h
-    const float ua = cubic_sqrt(fmaxf(n0 >= 0.0f ? t0 + e : t0 - e, 0.0f));
-    const float ub = cubic_sqrt(fmaxf(n1 >= 0.0f ? t1 - e : t1 + e, 0.0f));
+    // each end's own error: t is off by 2^-23 (4b^2 + |t|) at most.  (One error
+    // for both, the larger, lost forms within 10^-6 of a wide window's least end:
+    // where n < 0 the upper band takes the same roots, on the side that narrows
+    // it by e / 2t, and its factors allow for that only while e <= 3e-6 t; n < 0
+    // gives 4b^2 <= t.)
+    const float e0 = 1e-6f * (2.0f * fb2 + fabsf(t0)), e1 = 1e-6f * (2.0f * fb2 + fabsf(t1));
+    if (t0 + e0 < 0.0f) return B;  // the window lies above the largest h
+    const float ua = cubic_sqrt(fmaxf(n0 >= 0.0f ? t0 + e0 : t0 - e0, 0.0f));
+    const float ub = cubic_sqrt(fmaxf(n1 >= 0.0f ? t1 - e1 : t1 + e1, 0.0f));
     const float qs = fb * A.r3a;  // q*
     const float m = 1.0f + 2.5e-6f * P;
     // below q*: q = n / (2b + u)
     const float qa = n0 * cubic_rcp(fb + ua + 1e-30f);
-    const float qb = t1 > e ? n1 * cubic_rcp(fb + ub) : qs;
+    const float qb = t1 > e1 ? n1 * cubic_rcp(fb + ub) : qs;
     cubic_one_band(A, qa, qb, P, m + rho, m - rho, kres, sh, B.k[0], B.n[0]);
     // above q*: q = (2b + u) / (3a)
     if (qs <= 1.00001f)
