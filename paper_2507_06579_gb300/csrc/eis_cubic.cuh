@@ -148,8 +148,8 @@ EIS_HD float cubic_root(float g, float kappa) {
     return P;
 }
 
-// floor(x / m) and the remainder for |x| < 2^27, 8 < m < 2^15; rm = 1/m.
-// The estimate errs by less than 1 (|x/m| < 2^24), so one correction each way.
+// floor(x / m) and the remainder for |x| < 2^24, 3 <= m < 2^15; rm = 1/m rounded.
+// x is exact in fp32 and x rm errs by 2^-23 |x/m| < 1, so one correction each way.
 EIS_HD int32_t cubic_floordiv(int32_t x, int32_t m, float rm, int32_t &rem) {
     int32_t q = (int32_t)floorf((float)x * rm);
     int32_t r = x - q * m;
@@ -252,10 +252,10 @@ EIS_HD float cubic_rho(const CubicA &A, float fb, float fc, float &cq, float &q2
 
 // Forms of a band qlo <= q <= qhi: its first k and their number.
 EIS_HD void cubic_one_band(const CubicA &A, float qlo, float qhi, float P, float mlo, float mhi,
-                           int32_t kres, int32_t sh, int32_t &k0, int32_t &n) {
+                           uint32_t kres, int32_t sh, int32_t &k0, int32_t &n) {
     const int32_t lo = cubic_ceil((fmaxf(qlo, -1.0f) * P - mlo) * A.r9a);
     const int32_t hi = cubic_floor((fminf(qhi, 1.0f) * P + mhi) * A.r9a);
-    k0 = lo + ((kres - lo) & ((1 << sh) - 1));
+    k0 = lo + (int32_t)((kres - (uint32_t)lo) & ((1u << sh) - 1u));
     n = hi >= k0 ? ((hi - k0) >> sh) + 1 : 0;
 }
 
@@ -270,14 +270,15 @@ EIS_HD CubicBands cubic_bands(const CubicA &A, int32_t b, int32_t c) {
     const float P = cubic_fma(-fa, fc, fb1 * fb1);  // >= 1 (cubic_c_range)
     float cq, q2;
     const float rho = cubic_rho(A, fb1, fc, cq, q2);
-    // e == er mod the step  <=>  k == e0 - er
+    // e == er mod the step  <=>  k == e0 - er; only k's low bits count, so the bias
+    // 0x4B400000 of the two roundings' bits may stay, and the product may wrap
     const int32_t sh = cubic_shift(A.kind, a);
     int32_t er;
     if (A.kind)
         er = (a & b & 1) ? 0 : 1;
     else
         er = !(a & 1) ? 1 : (b & 1) ? 2 - a - b - c : 2;
-    const int32_t kres = b * (int32_t)float_bits(cq) + (int32_t)float_bits(q2) - er;
+    const uint32_t kres = (uint32_t)b * float_bits(cq) + float_bits(q2) - (uint32_t)er;
     // h(q) between n0 and n1; u = sqrt(4b^2 - 3a n) at either end, on the side
     // that widens n / (2b + u)
     const float ph = P * P, pl = cubic_fma(P, P, -ph), rp = cubic_rcp(ph);
