@@ -655,13 +655,23 @@ static int plan_build(eis_ctx *c, const uint64_t *lo, const uint64_t *hi, size_t
         p->tt.tau[0] = 1.39f / (float)c->mark_every;
         any_search = p->tt.nbaby[0] > 0;
     }
-    // cubic forms for the segments where they cost less than the walks they
-    // save; `left` is about what the queue will hold (all of a plain segment,
-    // at most 0.15 of a candidate's share where the forms decide: measured
-    // 0.09 to 0.11; with a log output all but the flagged)
-    uint64_t left = 0;
+    if (mode == EIS_MODE_PERSISTENT && c->giant_threshold > 0 && c->tune.empty() &&
+        c->giant_kernel == EIS_GIANT_WARP && p->total_cand > 0) {
+        giant_params(p->d_max, c->giant_stride, p->giant_nbaby, p->giant_log2n);
+        p->giant_log2n = std::min(p->giant_log2n, kGiantMaxLog2);
+        p->defer_after = (uint32_t)std::min<int64_t>(c->giant_threshold, 0xffffffffll);
+        p->defer_cap = (uint32_t)std::min<uint64_t>(p->total_cand, std::max<uint64_t>(1u << 16, p->total_cand / 4));
+        EIS_ALLOC(p->d_defer, (size_t)p->defer_cap * 4);
+        int occ = 0;
+        const size_t smem = (size_t)8 << p->giant_log2n;
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_giant, 32, smem) != cudaSuccess) {
+            cudaGetLastError();
+            occ = 1;
+        }
+        p->giant_grid = (uint32_t)(c->sm_count * std::max(1, occ));
+    }
+    // cubic forms for the segments where they cost less than the walks they save
     std::vector<uint8_t> segfield(nseg, 0);
-    uint64_t field_bytes = 0;
     if (mode == EIS_MODE_PERSISTENT && c->step_limit >= kCubicMinStepLimit) {
         double saved = 0;
         for (size_t si = 0; si < nseg; ++si) {
@@ -688,9 +698,41 @@ static int plan_build(eis_ctx *c, const uint64_t *lo, const uint64_t *hi, size_t
         if (units > 0xf0000000ull) p->cubic.clear();
         p->cubic_units = (uint32_t)units;
         p->cubic_grid = (uint32_t)std::min<uint64_t>((uint64_t)c->sm_count * c->occ_cubic, (units + 7) / 8);
-        if (!p->cubic.empty())
-            field_bytes = p->cubic.size() * sizeof(CubicJob) + nseg + 32 + (with_log ? 0 : p->nwords * 4);
     }
+    // The tables, and the forms' bitmap, before the search is sized: it takes
+    // what room is left.  Without room for theirs the plan does without the forms.
+    std::vector<unsigned char> tab;
+    for (;;) {
+        const size_t o_tiles = nseg * sizeof(Seg), o_cubic = o_tiles + ntiles * sizeof(Tile),
+                     o_field = o_cubic + p->cubic.size() * sizeof(CubicJob);
+        rc = plan_alloc(p, (void **)&p->d_tab, o_field + nseg);
+        if (rc != EIS_OK && !p->cubic.empty()) {
+            p->cubic.clear();
+            continue;
+        }
+        if (rc != EIS_OK) {
+            plan_free(p);
+            return rc;
+        }
+        tab.resize(o_field + nseg);
+        if (nseg) std::memcpy(tab.data(), p->segs.data(), nseg * sizeof(Seg));
+        if (ntiles) std::memcpy(tab.data() + o_tiles, p->tiles.data(), ntiles * sizeof(Tile));
+        if (!p->cubic.empty())
+            std::memcpy(tab.data() + o_cubic, p->cubic.data(), p->cubic.size() * sizeof(CubicJob));
+        if (nseg) std::memcpy(tab.data() + o_field, segfield.data(), nseg);
+        p->d_segs = reinterpret_cast<Seg *>(p->d_tab);
+        p->d_tiles = reinterpret_cast<Tile *>(p->d_tab + o_tiles);
+        p->d_cubic = reinterpret_cast<CubicJob *>(p->d_tab + o_cubic);
+        p->d_segfield = p->d_tab + o_field;
+        break;
+    }
+    if (!p->cubic.empty() && !with_log &&
+        plan_alloc(p, (void **)&p->d_field, p->nwords * 4) != EIS_OK)
+        p->cubic.clear();
+    // `left` is about what the queue will hold (all of a plain segment, at most
+    // 0.15 of a candidate's share where the forms decide: measured 0.09 to 0.11;
+    // with a log output all but the flagged)
+    uint64_t left = 0;
     uint64_t left_walk = 0;  // of which of segments that the forms do not decide
     for (size_t si = 0; si < nseg; ++si) {
         const bool plain = p->cubic.empty() || !segfield[si] || with_log;
@@ -716,7 +758,7 @@ static int plan_build(eis_ctx *c, const uint64_t *lo, const uint64_t *hi, size_t
         const uint64_t per_d = kBsgsRegionBytes + sizeof(DRecord) + 4;
         const uint64_t used = c->in_use.load();
         const uint64_t cached = pool_cached_bytes(c);  // reclaimable
-        const uint64_t room = c->budget + cached > used + field_bytes ? c->budget + cached - used - field_bytes : 0;
+        const uint64_t room = c->budget + cached > used ? c->budget + cached - used : 0;
         const uint64_t fit = room / per_d > lanes + 64 ? room / per_d - lanes - 64 : 0;
         uint64_t C = std::min<uint64_t>((uint64_t)c->bsgs_chunk, queue);
         // (for callers who never asked for the search its tables take a
@@ -754,47 +796,14 @@ static int plan_build(eis_ctx *c, const uint64_t *lo, const uint64_t *hi, size_t
             EIS_ALLOC(p->d_bctr, 8 * sizeof(uint32_t));
             p->bev.assign(3 * (size_t)p->bsgs_rounds, nullptr);
         }
-    } else if (mode == EIS_MODE_PERSISTENT && c->giant_threshold > 0 && c->tune.empty() &&
-               c->giant_kernel == EIS_GIANT_WARP && p->total_cand > 0) {
-        giant_params(p->d_max, c->giant_stride, p->giant_nbaby, p->giant_log2n);
-        p->giant_log2n = std::min(p->giant_log2n, kGiantMaxLog2);
-        p->defer_after = (uint32_t)std::min<int64_t>(c->giant_threshold, 0xffffffffll);
-        p->defer_cap = (uint32_t)std::min<uint64_t>(p->total_cand, std::max<uint64_t>(1u << 16, p->total_cand / 4));
-        EIS_ALLOC(p->d_defer, (size_t)p->defer_cap * 4);
-        int occ = 0;
-        const size_t smem = (size_t)8 << p->giant_log2n;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_giant, 32, smem) != cudaSuccess) {
-            cudaGetLastError();
-            occ = 1;
-        }
-        p->giant_grid = (uint32_t)(c->sm_count * std::max(1, occ));
     }
-    {
-        const size_t o_tiles = nseg * sizeof(Seg), o_cubic = o_tiles + ntiles * sizeof(Tile),
-                     o_field = o_cubic + p->cubic.size() * sizeof(CubicJob);
-        std::vector<unsigned char> h(o_field + nseg);
-        if (nseg) std::memcpy(h.data(), p->segs.data(), nseg * sizeof(Seg));
-        if (ntiles) std::memcpy(h.data() + o_tiles, p->tiles.data(), ntiles * sizeof(Tile));
-        if (!p->cubic.empty())
-            std::memcpy(h.data() + o_cubic, p->cubic.data(), p->cubic.size() * sizeof(CubicJob));
-        if (nseg) std::memcpy(h.data() + o_field, segfield.data(), nseg);
-        EIS_ALLOC(p->d_tab, h.size());
-        p->d_segs = reinterpret_cast<Seg *>(p->d_tab);
-        p->d_tiles = reinterpret_cast<Tile *>(p->d_tab + o_tiles);
-        p->d_cubic = reinterpret_cast<CubicJob *>(p->d_tab + o_cubic);
-        p->d_segfield = p->d_tab + o_field;
-        // (the stream's allocations are complete, and the copy done, after the wait)
-        if ((!h.empty() && cudaMemcpyAsync(p->d_tab, h.data(), h.size(), cudaMemcpyHostToDevice,
-                                           c->aux) != cudaSuccess) ||
-            cudaStreamSynchronize(c->aux) != cudaSuccess) {
-            plan_free(p);
-            return EIS_EDEVICE;
-        }
+    // (the last allocation: the stream's are complete, and the copy done, after the wait)
+    if ((!tab.empty() && cudaMemcpyAsync(p->d_tab, tab.data(), tab.size(), cudaMemcpyHostToDevice,
+                                         c->aux) != cudaSuccess) ||
+        cudaStreamSynchronize(c->aux) != cudaSuccess) {
+        plan_free(p);
+        return EIS_EDEVICE;
     }
-    // without room for its bitmap the plan does without the forms
-    if (!p->cubic.empty() && !with_log &&
-        plan_alloc(p, (void **)&p->d_field, p->nwords * 4) != EIS_OK)
-        p->cubic.clear();
 #undef EIS_ALLOC
     // Few d, all walked: they fit the GPU at once, one thread each, and the queue
     // (a scan, a compaction) would only come before the walk.  [5, 10^6]: 57 us

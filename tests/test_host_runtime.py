@@ -1,0 +1,96 @@
+"""Host side of plans and calls (allocation, ordering between streams, memory
+budget), over a CUDA runtime without a device (fakert.py)."""
+import pytest
+
+import fakert
+import paper_2507_06579_gb300 as E
+
+
+@pytest.fixture()
+def rt():
+    with fakert.installed() as L:
+        yield L
+
+
+@pytest.mark.parametrize("flags", [0, E.EIS_PLAN_CLASSES, E.EIS_PLAN_PRIMES])
+@pytest.mark.parametrize("thr", [0, 1024])
+def test_a_plans_buffers_are_waited_for_before_other_streams_use_them(rt, flags, thr):
+    """Buffers are allocated in the order of the context's own stream: the plan
+    waits for every one of them before its launches, on any stream, use it."""
+    with E.Context(0) as c:
+        c.set_option(E.EIS_OPT_GIANT_THRESHOLD, thr)
+        for stream in (None, 12345):
+            p = c.plan_create([10**9, 10**10], [10**9 + 10**8, 10**10 + 10**8], E.EIS_MODE_PERSISTENT, flags)
+            p.launch(stream)
+            p.counts()
+            p.destroy()
+        assert rt.fake_launches(b"k_cubic") > 0  # the forms' bitmap is one of them
+        c.count_range(10**9, 10**9 + 10**8)
+        c.classify_range_u8(10**9, 10**9 + 10**8)
+    assert rt.fake_violations() == 0
+
+
+def _plan(rt, c, n=1 << 23):
+    """Kernels of one launch of a plan of n candidates, or None if it is refused."""
+    try:
+        p = c.plan_create([10**9], [10**9 + 8 * n])
+    except E.EisError as e:
+        assert e.code == E.EIS_ENOMEM
+        return None
+    rt.fake_fail_after(-1)
+    p.launch()
+    p.counts()
+    p.destroy()
+    return {k: rt.fake_launches(k.encode()) for k in ("k_cubic", "k_walk_record", "k_walk_persistent")}
+
+
+def test_a_plan_that_loses_the_forms_is_sized_for_all_its_d(rt):
+    """Where the memory for the forms' bitmap cannot be had, the search's rounds
+    are those of a plan that never had the forms (they were those of 15% of the
+    d, and the last round walked the rest)."""
+    def context():
+        c = E.Context(0)
+        c.set_option(E.EIS_OPT_USE_GRAPH, 0)
+        c.set_option(E.EIS_OPT_GIANT_THRESHOLD, 1024)
+        c.set_option(E.EIS_OPT_BSGS_CHUNK, 1 << 20)
+        return c
+
+    with context() as c:
+        c.set_option(E.EIS_OPT_STEP_LIMIT, 1 << 25)  # no forms
+        rt.fake_reset()
+        without = _plan(rt, c)
+    assert without["k_cubic"] == 0 and without["k_walk_record"] == 8
+    lost = 0
+    for n in range(16):
+        with context() as c:
+            rt.fake_reset()
+            rt.fake_fail_after(n)
+            got = _plan(rt, c)
+            if got and not got["k_cubic"]:
+                assert got == without
+                lost += 1
+    assert lost > 0
+
+
+def test_the_warp_search_keeps_its_list_in_a_tight_budget(rt):
+    """A budget that holds the plan with the warp search's list but not the
+    forms' bitmap: the plan is made, without the forms."""
+    def need(limit):
+        with E.Context(0) as c:
+            c.set_option(E.EIS_OPT_STEP_LIMIT, limit)
+            return used(c)
+
+    def used(c):
+        c.set_option(E.EIS_OPT_GIANT_KERNEL, E.EIS_GIANT_WARP)
+        c.set_option(E.EIS_OPT_GIANT_THRESHOLD, 32768)
+        p = c.plan_create([10**9], [10**9 + (8 << 20)])
+        n = c.get_option(E.EIS_OPT_MEM_IN_USE)
+        p.launch()
+        p.destroy()
+        return n
+
+    with_forms, without = need(1 << 26), need(1 << 25)
+    assert with_forms > without + (1 << 17) - 1  # the bitmap
+    with E.Context(0, mem_budget_bytes=with_forms - (1 << 16)) as c:
+        rt.fake_reset()
+        assert used(c) < with_forms and rt.fake_launches(b"k_cubic") == 0
