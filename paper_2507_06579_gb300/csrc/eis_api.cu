@@ -203,6 +203,16 @@ static int plan_alloc(eis_plan *p, void **ptr, size_t bytes, bool own = false) {
     return EIS_ENOMEM;
 }
 
+// Give a buffer of plan_alloc back (null: nothing).
+template <class T>
+static void plan_unalloc(eis_plan *p, T *&ptr, size_t bytes) {
+    if (!ptr) return;
+    cudaFreeAsync(ptr, p->ctx->aux);
+    ctx_release(p->ctx, bytes);
+    p->bytes -= bytes;
+    ptr = nullptr;
+}
+
 // The cached search pool if it holds at least `bytes` (its charge moves to the
 // caller, *got = its size); a smaller one is freed.  nullptr if none fits.
 static unsigned char *pool_take(eis_ctx *c, uint64_t bytes, uint64_t *got) {
@@ -343,6 +353,10 @@ static constexpr int kGiantMaxLog2 = 14;  // 128 KB table per warp at most
 static constexpr uint32_t kGiantMaxRounds = 1u << 20;
 static constexpr double kTuneMargin = 0.98;  // autotuner: keep the current setting unless 2% faster
 static constexpr uint32_t kBsgsMaxCycles = 1u << 20;  // giant cycles per d before the fallback walk
+
+// From this many candidates on, a plan whose options ask for the search is
+// refused when its tables cannot be had; a smaller one walks.
+static constexpr uint64_t kSearchMustCands = (uint64_t)1 << 18;
 
 // Plans of at most this many candidates and no search run the plain walk.
 static constexpr uint64_t kPlainMaxCands = (uint64_t)1 << 17;
@@ -780,21 +794,32 @@ static int plan_build(eis_ctx *c, const uint64_t *lo, const uint64_t *hi, size_t
             if (p->d_pool) {
                 p->pool_bytes = got;  // its charge moves to this plan
                 p->bytes += got;
-            } else if (plan_alloc(p, (void **)&p->d_pool, pool_need, true) == EIS_OK) {
-                p->pool_bytes = pool_need;
-            } else if (own) {
-                p->bsgs = 0;  // nobody asked for the search: the plan walks
-                p->d_pool = nullptr;
+                rc = EIS_OK;
+            } else {
+                rc = plan_alloc(p, (void **)&p->d_pool, pool_need, true);
+                if (rc == EIS_OK) p->pool_bytes = pool_need;
+            }
+            if (rc == EIS_OK) rc = plan_alloc(p, (void **)&p->d_recs, C * sizeof(DRecord));
+            if (rc == EIS_OK) rc = plan_alloc(p, (void **)&p->d_fb, C * 4);
+            if (rc == EIS_OK) rc = plan_alloc(p, (void **)&p->d_bctr, 8 * sizeof(uint32_t));
+            if (rc == EIS_OK) {
+                p->bev.assign(3 * (size_t)p->bsgs_rounds, nullptr);
+            } else if (own || p->total_cand < kSearchMustCands) {
+                // nobody asked for the search: the plan walks
+                p->bsgs = 0;
+                if (p->d_pool) {
+                    cudaFree(p->d_pool);
+                    ctx_release(c, p->pool_bytes);
+                    p->bytes -= p->pool_bytes;
+                    p->d_pool = nullptr;
+                    p->pool_bytes = 0;
+                }
+                plan_unalloc(p, p->d_recs, C * sizeof(DRecord));
+                plan_unalloc(p, p->d_fb, C * 4);
             } else {
                 plan_free(p);
-                return EIS_ENOMEM;
+                return rc;
             }
-        }
-        if (p->bsgs) {
-            EIS_ALLOC(p->d_recs, C * sizeof(DRecord));
-            EIS_ALLOC(p->d_fb, C * 4);
-            EIS_ALLOC(p->d_bctr, 8 * sizeof(uint32_t));
-            p->bev.assign(3 * (size_t)p->bsgs_rounds, nullptr);
         }
     }
     // (the last allocation: the stream's are complete, and the copy done, after the wait)

@@ -8,7 +8,7 @@
 //  * bytes mapped: cudaMalloc's, and what the memory pools hold (freed blocks
 //    stay until a wait, above the release threshold, or cudaMemPoolTrimTo), the
 //    highest value since the last reset, and a capacity past which allocations
-//    fail; the n-th allocation from now on can be made to fail;
+//    fail; the n-th allocation from now on, and some after it, can be made to fail;
 //  * waits, graph launches, and whether a stream is capturing.
 #include <cuda_runtime.h>
 #include <sys/mman.h>
@@ -39,7 +39,7 @@ std::map<const void *, std::string> names;
 std::map<std::string, long> launches;
 std::set<cudaStream_t> capturing;
 size_t malloced = 0, capacity = (size_t)200 << 30, peak = 0;
-long violations = 0, fail_after = -1, next_id = 1, waits = 0;
+long violations = 0, fail_after = -1, fail_count = 0, next_id = 1, waits = 0;
 dim3 cfg_grid, cfg_block;
 size_t cfg_smem;
 cudaStream_t cfg_stream;
@@ -58,7 +58,8 @@ cudaError_t fail(cudaError_t e) {
 
 // Whether an allocation that maps `more` bytes succeeds.
 bool room(size_t more) {
-    if (fail_after >= 0 && fail_after-- == 0) return false;
+    if (fail_after > 0) --fail_after;
+    else if (fail_after == 0 && fail_count > 0) { --fail_count; return false; }
     if (mapped() + more > capacity) return false;
     return true;
 }
@@ -105,7 +106,7 @@ long fake_waits() { LOCK; return waits; }
 unsigned long long fake_mapped() { LOCK; return mapped(); }
 unsigned long long fake_peak() { LOCK; return peak; }
 void fake_set_capacity(unsigned long long b) { LOCK; capacity = b; }
-void fake_fail_after(long n) { LOCK; fail_after = n; }
+void fake_fail_after(long n, long count) { LOCK; fail_after = n; fail_count = count; }
 void fake_capture(void *s, int on) { LOCK; if (on) capturing.insert((cudaStream_t)s); else capturing.erase((cudaStream_t)s); }
 void fake_reset() {
     LOCK;

@@ -34,7 +34,7 @@ def load():
         L.fake_launches.restype = L.fake_violations.restype = L.fake_waits.restype = ctypes.c_long
         L.fake_mapped.restype = L.fake_peak.restype = ctypes.c_ulonglong
         L.fake_set_capacity.argtypes = [ctypes.c_ulonglong]
-        L.fake_fail_after.argtypes = [ctypes.c_long]
+        L.fake_fail_after.argtypes = [ctypes.c_long, ctypes.c_long]
         L.fake_capture.argtypes = [ctypes.c_void_p, ctypes.c_int]
         _fake = L
     return _fake
@@ -50,6 +50,6 @@ def installed():
     try:
         yield L
     finally:
-        L.fake_fail_after(-1)
+        L.fake_fail_after(-1, 0)
         L.fake_set_capacity(200 << 30)
         E._lib = saved

@@ -37,7 +37,7 @@ def _plan(rt, c, n=1 << 23):
     except E.EisError as e:
         assert e.code == E.EIS_ENOMEM
         return None
-    rt.fake_fail_after(-1)
+    rt.fake_fail_after(-1, 0)
     p.launch()
     p.counts()
     p.destroy()
@@ -64,7 +64,7 @@ def test_a_plan_that_loses_the_forms_is_sized_for_all_its_d(rt):
     for n in range(16):
         with context() as c:
             rt.fake_reset()
-            rt.fake_fail_after(n)
+            rt.fake_fail_after(n, 1)
             got = _plan(rt, c)
             if got and not got["k_cubic"]:
                 assert got == without
@@ -94,3 +94,32 @@ def test_the_warp_search_keeps_its_list_in_a_tight_budget(rt):
     with E.Context(0, mem_budget_bytes=with_forms - (1 << 16)) as c:
         rt.fake_reset()
         assert used(c) < with_forms and rt.fake_launches(b"k_cubic") == 0
+
+
+@pytest.mark.parametrize("thr,n", [(0, 1 << 22), (0, 1 << 17), (1024, 1 << 17)])
+def test_without_memory_for_the_searchs_tables_the_plan_walks(rt, thr, n):
+    """Callers who did not ask for the search, and small plans, are refused only
+    for the buffers a walk needs: two bitmaps, two words a tile, the queue, the
+    results and the tables."""
+    refused, walked = 0, 0
+    for i in range(16):
+        with E.Context(0) as c:
+            c.set_option(E.EIS_OPT_GIANT_THRESHOLD, thr)
+            used0 = c.get_option(E.EIS_OPT_MEM_IN_USE)
+            rt.fake_reset()
+            rt.fake_fail_after(i, 4)
+            try:
+                p = c.plan_create([10**12], [10**12 + 8 * n])
+            except E.EisError as e:
+                assert e.code == E.EIS_ENOMEM
+                refused += 1
+                p = None
+            rt.fake_fail_after(-1, 0)
+            if p:
+                p.launch()
+                p.counts()
+                walked += rt.fake_launches(b"k_walk_record") == 0
+                p.destroy()
+            cached = c.get_option(E.EIS_OPT_MEM_IN_USE) - used0
+            assert cached == 0 or rt.fake_launches(b"k_walk_record") > 0  # the kept pool
+    assert refused == 7 and walked > 0
