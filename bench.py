@@ -252,7 +252,7 @@ def main():
     ap.add_argument("--window", type=float, default=WINDOW,
                     help="per-rank window width below 1e11 (smaller for profiling runs)")
     ap.add_argument("--nbaby", type=int, default=0,
-                    help="with --no-autotune: lane search after this many baby steps (0: walk only)")
+                    help="with --no-autotune: lane search after this many baby steps (0: the library's own settings)")
     ap.add_argument("--mark-every", type=int, default=32,
                     help="with --nbaby: about 1 state in this many is marked")
     ap.add_argument("--bsgs-chunk", type=int, default=0,

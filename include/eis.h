@@ -84,9 +84,10 @@ extern "C" {
 #define EIS_OPT_STEP_LIMIT 4     /* per-d baby-step limit before EIS_ESTEPS   */
 #define EIS_OPT_USE_GRAPH 5      /* 1: capture plans into CUDA graphs (1)     */
 #define EIS_OPT_GIANT_THRESHOLD 6 /* baby steps after which a d is handed to  */
-                                  /* the giant-step kernel (0, the default:   */
+                                  /* the giant-step kernel.  0, the default:  */
                                   /* the library's own choice by d; never,    */
-                                  /* with EIS_OPT_STEP_LIMIT below 2^26)      */
+                                  /* with EIS_OPT_GIANT_KERNEL EIS_GIANT_WARP */
+                                  /* or EIS_OPT_STEP_LIMIT below 2^26         */
 #define EIS_OPT_GIANT_STRIDE 7   /* giant-step stride in baby steps (0: auto) */
 #define EIS_OPT_GIANT_COMPOSE 8  /* giant-step composition: EIS_COMPOSE_*      */
 #define EIS_OPT_MEM_BUDGET 9     /* read-only: the context's device-memory    */
@@ -231,7 +232,8 @@ int eis_count_batch(eis_ctx *ctx, const uint64_t *lo, const uint64_t *hi, size_t
 typedef struct {
     int32_t ctas_per_sm;     /* persistent walk CTAs per SM chosen */
     int64_t giant_threshold; /* baby steps before a walk goes to a giant-step  */
-                             /* search (0: never)                               */
+                             /* search (0: with EIS_GIANT_WARP never, with      */
+                             /* EIS_GIANT_LANE the library's own choice by d)   */
     int64_t giant_stride;    /* warp-per-d search: baby count N (0: automatic)  */
     double ms_best;          /* device time of one pass with the chosen setting */
     double ms_default;       /* ... and with the context's previous setting     */
@@ -274,9 +276,10 @@ int eis_autotune_decades(eis_ctx *ctx, uint64_t d_lo, uint64_t d_hi, eis_tune_ro
 
 /* Time candidate settings on the sample [lo, hi) -- a window of the d-range
  * the context will serve -- with any tuning table set aside: CTAs per SM of
- * the persistent walk; threads per d (the walk alone, the lane search at one
- * thread per d, or the warp-per-d kernel at 32 with its threshold); and the
- * lane search's round size (chunk of survivors).  The fastest stays in the
+ * the persistent walk (timed on the walk alone); the library's own settings;
+ * threads per d (the lane search at one thread per d, or the warp-per-d kernel
+ * at 32 with its threshold); and the lane search's round size (chunk of
+ * survivors).  The fastest stays in the
  * context, provided it beats the previous setting by more than 2% (else the
  * previous stays); the table is restored.  Every candidate runs a full plan
  * (sieve, walks, count); results are identical for every setting, only time

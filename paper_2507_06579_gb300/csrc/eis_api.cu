@@ -650,10 +650,11 @@ static int plan_build(eis_ctx *c, const uint64_t *lo, const uint64_t *hi, size_t
     if (flags & EIS_PLAN_CLASSES) p->d_cls = p->d_counts + 2 * nseg + 1;
     if (with_log) EIS_ALLOC(p->d_glog, p->total_cand);
     // the settings each d of the plan takes: the context's tuning table, or
-    // one row of EIS_OPT_GIANT_THRESHOLD / EIS_OPT_MARK_EVERY, or (threshold 0,
-    // at a step limit no walk reaches) the library's own
+    // one row of EIS_OPT_GIANT_THRESHOLD / EIS_OPT_MARK_EVERY, or (threshold 0 of
+    // the lane search, at a step limit no walk reaches) the library's own
     bool any_search = false;
-    const bool own = c->tune.empty() && c->giant_threshold == 0 && c->step_limit >= kCubicMinStepLimit;
+    const bool own = c->tune.empty() && c->giant_kernel == EIS_GIANT_LANE && c->giant_threshold == 0 &&
+                     c->step_limit >= kCubicMinStepLimit;
     if (own) {
         auto_rows(p->tt, false, 0, 0);
         for (const Seg &sg : p->segs)
@@ -1517,10 +1518,11 @@ int eis_autotune(eis_ctx *c, uint64_t lo, uint64_t hi, eis_tune_result *out) {
     EisNvtxRange range("eis.autotune");
     if (!c || !out || lo >= hi) return EIS_EINVAL;
     if (hi > EIS_D_LIMIT) return EIS_ERANGE;
-    // CTAs per SM of the walk; threads per d (0 = walk only, the lane search
-    // at 1 thread per d, the warp-per-d kernel at 32) with its threshold;
-    // and the round size of the lane search (the chunk of survivors whose
-    // tables one round holds)
+    // CTAs per SM of the walk, timed on the walk alone (EIS_GIANT_WARP with
+    // threshold 0: no search, so that the walk's kernel takes every d); the
+    // library's own settings (EIS_GIANT_LANE with threshold 0); the
+    // warp-per-d kernel with its threshold; and the round size of the lane
+    // search (the chunk of survivors whose tables one round holds)
     struct Setting {
         int ctas;
         int kernel;
@@ -1529,7 +1531,8 @@ int eis_autotune(eis_ctx *c, uint64_t lo, uint64_t hi, eis_tune_result *out) {
     const int occ = c->occ_persistent;
     std::vector<Setting> cands;
     for (int ctas : {occ, std::max(1, occ * 3 / 4), std::max(1, occ / 2)})
-        cands.push_back({ctas, EIS_GIANT_LANE, 0, c->bsgs_chunk});
+        cands.push_back({ctas, EIS_GIANT_WARP, 0, c->bsgs_chunk});
+    cands.push_back({occ, EIS_GIANT_LANE, 0, c->bsgs_chunk});
     for (int64_t thr : {(int64_t)32768, (int64_t)131072})
         cands.push_back({occ, EIS_GIANT_WARP, thr, c->bsgs_chunk});
     const int64_t lane_thr = c->giant_kernel == EIS_GIANT_LANE && c->giant_threshold > 0

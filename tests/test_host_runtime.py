@@ -123,3 +123,20 @@ def test_without_memory_for_the_searchs_tables_the_plan_walks(rt, thr, n):
             cached = c.get_option(E.EIS_OPT_MEM_IN_USE) - used0
             assert cached == 0 or rt.fake_launches(b"k_walk_record") > 0  # the kept pool
     assert refused == 7 and walked > 0
+
+
+def test_the_autotuner_times_the_walk(rt):
+    """Three of its trials (the CTA counts) walk every d that the forms leave:
+    no trial differs by a setting that its kernels do not use."""
+    with E.Context(0) as c:
+        rt.fake_reset()
+        trials = c.autotune(10**11, 10**11 + (8 << 20))["trials"]
+        plans, searched, warp = (rt.fake_launches(k) for k in (b"k_scan_tiles", b"k_walk_record", b"k_giant"))
+        assert plans == trials and searched >= 6 and warp == 2
+        assert plans - searched - warp == 3
+        # and the walk alone can be asked for
+        c.set_option(E.EIS_OPT_GIANT_KERNEL, E.EIS_GIANT_WARP)
+        assert c.get_option(E.EIS_OPT_GIANT_THRESHOLD) == 0
+        rt.fake_reset()
+        c.count_range(10**11, 10**11 + (8 << 20))
+        assert rt.fake_launches(b"k_walk_persistent") == 1 and rt.fake_launches(b"k_walk_record") == 0
