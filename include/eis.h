@@ -156,7 +156,10 @@ typedef struct {
  * ------------------------------------------------------------------- */
 
 /* Create a context on CUDA device `device`.  mem_budget_bytes bounds the
- * device memory the context and its plans may hold (0: 3/4 of free memory).
+ * device memory the context, its plans and its servers may hold (0: 3/4 of free
+ * memory).  Between plans the context keeps up to 1 GB of their freed buffers
+ * mapped (inside the budget, not in EIS_OPT_MEM_IN_USE), and one lane-search
+ * table pool (in EIS_OPT_MEM_IN_USE); both give way to what is asked for next.
  * Builds the odd-prime table up to 2^22 (for the square-free sieve of d <
  * 2^44) on the device.  *out receives the context. */
 int eis_create(eis_ctx **out, int device, uint64_t mem_budget_bytes);

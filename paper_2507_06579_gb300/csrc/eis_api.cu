@@ -58,7 +58,9 @@ struct eis_ctx {
     // Plans' buffers come from this memory pool, which keeps up to
     // kMempoolKeep freed bytes mapped: with cudaMalloc and cudaFree (a dozen a
     // plan) a call over a short range spent most of its time on them.
+    // (They count against the budget: mempool_fit.)
     cudaMemPool_t mempool = nullptr;
+    uint64_t in_use_peak = 0;
     cudaStream_t aux = nullptr;      // allocations and table copies (never behind a launch)
     unsigned char *h_res = nullptr;  // pinned: a plan's results on their way to the host
     unsigned char *pool_cache = nullptr;
@@ -181,6 +183,31 @@ static void ctx_release(eis_ctx *c, uint64_t bytes) {
     }
 }
 
+// Give what the memory pool keeps mapped back to the device.
+static void mempool_trim(eis_ctx *c) {
+    cudaStreamSynchronize(c->aux);  // plans' buffers are freed in its order
+    cudaMemPoolTrimTo(c->mempool, 0);
+}
+
+// The budget bounds what is mapped: before `bytes` more are (charged already;
+// of_pool: they may come out of what the pool keeps), the pool gives back what
+// it keeps if it would not fit beside them.  (The pool holds at most about what
+// was ever charged, so that contexts far from their budget need not ask it.)
+static void mempool_fit(eis_ctx *c, uint64_t bytes, bool of_pool) {
+    const uint64_t used = c->in_use.load();
+    c->in_use_peak = std::max(c->in_use_peak, used);
+    if (used + 2 * c->in_use_peak <= c->budget) return;
+    uint64_t held = 0, live = 0;
+    if (cudaMemPoolGetAttribute(c->mempool, cudaMemPoolAttrReservedMemCurrent, &held) != cudaSuccess ||
+        cudaMemPoolGetAttribute(c->mempool, cudaMemPoolAttrUsedMemCurrent, &live) != cudaSuccess) {
+        cudaGetLastError();
+        return;
+    }
+    uint64_t kept = held > live ? held - live : 0;
+    if (of_pool) kept -= std::min(kept, bytes);
+    if (used + kept > c->budget) mempool_trim(c);
+}
+
 // Device memory for a plan, charged to the context: from its memory pool in
 // the order of its aux stream (plan_build waits for it before it returns),
 // or, for the search's tables, mapped on its own.
@@ -188,7 +215,8 @@ static int plan_alloc(eis_plan *p, void **ptr, size_t bytes, bool own = false) {
     if (bytes == 0) bytes = 16;
     eis_ctx *c = p->ctx;
     if (!ctx_reserve(c, bytes)) return EIS_ENOMEM;
-    for (int t = 0; t < 2; ++t) {
+    mempool_fit(c, bytes, !own);
+    for (int t = 0; t < 3; ++t) {
         const cudaError_t e = own ? cudaMalloc(ptr, bytes)
                                   : cudaMallocFromPoolAsync(ptr, bytes, c->mempool, c->aux);
         if (e == cudaSuccess) {
@@ -197,7 +225,10 @@ static int plan_alloc(eis_plan *p, void **ptr, size_t bytes, bool own = false) {
         }
         cudaGetLastError();
         *ptr = nullptr;
-        if (!pool_drop(c)) break;
+        if (t == 0)
+            mempool_trim(c);
+        else if (!pool_drop(c))
+            break;
     }
     ctx_release(c, bytes);
     return EIS_ENOMEM;
@@ -1048,7 +1079,16 @@ void eis_giant_params(uint64_t d, int64_t forced, int &nbaby, int &log2n) {
     log2n = std::min(log2n, kGiantMaxLog2);
 }
 
-bool eis_ctx_reserve(eis_ctx *c, uint64_t bytes) { return ctx_reserve(c, bytes); }
+bool eis_ctx_reserve(eis_ctx *c, uint64_t bytes) {
+    if (!ctx_reserve(c, bytes)) return false;
+    mempool_fit(c, bytes, false);
+    return true;
+}
+
+void eis_ctx_trim(eis_ctx *c) {
+    mempool_trim(c);
+    pool_drop(c);
+}
 
 void eis_ctx_release(eis_ctx *c, uint64_t bytes) { ctx_release(c, bytes); }
 
@@ -1658,9 +1698,12 @@ int eis_classify_range_u8(eis_ctx *c, uint64_t lo, uint64_t hi, uint8_t *codes_o
         if (n == 0) return EIS_OK;
         uint8_t *tmp = out_on_device ? codes_out + off : nullptr;
         if (!tmp) {
-            if (cudaMallocFromPoolAsync(reinterpret_cast<void **>(&tmp), n, c->mempool, s) != cudaSuccess) {
+            for (int t = 0;; ++t) {
+                if (cudaMallocFromPoolAsync(reinterpret_cast<void **>(&tmp), n, c->mempool, s) == cudaSuccess)
+                    break;
                 cudaGetLastError();
-                return EIS_ENOMEM;
+                if (t) return EIS_ENOMEM;
+                eis_ctx_trim(c);
             }
         }
         const uint32_t grid = (uint32_t)std::min<uint64_t>((n + 255) / 256, 65535ull * 8);

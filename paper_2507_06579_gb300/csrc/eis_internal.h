@@ -41,6 +41,8 @@ uint32_t eis_ctx_primes_up_to(eis_ctx *ctx, uint64_t d);
 // Account `bytes` of device memory against the context budget; false if over.
 bool eis_ctx_reserve(eis_ctx *ctx, uint64_t bytes);
 void eis_ctx_release(eis_ctx *ctx, uint64_t bytes);
+// Give back to the device what the context keeps mapped for its next plan.
+void eis_ctx_trim(eis_ctx *ctx);
 
 // Host-side NVTX range for the phases a profiler timeline should show
 // (plan build and launch, single queries, autotuning, server batches).  The

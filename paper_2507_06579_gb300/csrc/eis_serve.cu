@@ -538,6 +538,10 @@ int eis_server_create(eis_ctx *ctx, const eis_server_config *cfg, eis_server **o
         return rc;
     };
     int rc = alloc_slots();
+    if (rc == EIS_ENOMEM) {  // what the context keeps for its plans gives way
+        eis_ctx_trim(ctx);
+        rc = alloc_slots();
+    }
     if (rc == EIS_ENOMEM && s->search_chunk) {  // without the search's tables, then
         const uint64_t more = search_bytes(s->search_chunk, s->rec_grid) * c.slots;
         eis_ctx_release(ctx, more);

@@ -64,7 +64,7 @@ def test_a_plan_that_loses_the_forms_is_sized_for_all_its_d(rt):
     for n in range(16):
         with context() as c:
             rt.fake_reset()
-            rt.fake_fail_after(n, 1)
+            rt.fake_fail_after(n, 2)
             got = _plan(rt, c)
             if got and not got["k_cubic"]:
                 assert got == without
@@ -140,3 +140,46 @@ def test_the_autotuner_times_the_walk(rt):
         rt.fake_reset()
         c.count_range(10**11, 10**11 + (8 << 20))
         assert rt.fake_launches(b"k_walk_persistent") == 1 and rt.fake_launches(b"k_walk_record") == 0
+
+
+def test_mapped_memory_stays_within_the_budget(rt):
+    """Freed buffers that the context keeps mapped count: a plan's search tables
+    and a server's slots are not mapped beside them past the budget."""
+    budget = 192 << 20
+    with E.Context(0, mem_budget_bytes=budget) as c:
+        rt.fake_reset()
+        walk, search = [(E.EIS_D_LIMIT, 0, 16)], [(E.EIS_D_LIMIT, 512, 16)]
+        for rows, n in ((walk, 30 << 20), (search, 1 << 16), (walk, 30 << 20), (walk, 1 << 10)):
+            c.set_tune_table(rows)
+            p = c.plan_create([10**9], [10**9 + 8 * n])
+            p.launch()
+            p.counts()
+            searched = rt.fake_launches(b"k_walk_record") > 0
+            p.destroy()
+        assert searched
+        with E.Server(c, slots=4, slot_candidates=1 << 22):
+            pass
+        assert (128 << 20) < rt.fake_peak() <= budget
+
+
+def test_kept_memory_gives_way_where_the_device_has_no_more(rt):
+    """An allocation that the device refuses is tried again without what the
+    context keeps mapped: plan buffers, search tables, a server's slots."""
+    def grown(c):
+        c.set_tune_table([(E.EIS_D_LIMIT, 0, 16)])
+        p = c.plan_create([10**9], [10**9 + 8 * (200 << 20)])
+        p.launch()
+        p.counts()
+        p.destroy()
+        rt.fake_set_capacity(rt.fake_mapped() + (1 << 20))  # someone else has the rest
+
+    with E.Context(0) as c:
+        grown(c)
+        c.set_tune_table([(E.EIS_D_LIMIT, 512, 16)])
+        p = c.plan_create([10**12], [10**12 + (8 << 18)])  # refused before
+        p.destroy()
+    rt.fake_set_capacity(200 << 30)
+    with E.Context(0) as c:
+        grown(c)
+        with E.Server(c, slots=1, slot_candidates=1 << 16, giant_after=131072) as srv:  # refused before
+            srv.stats()
