@@ -408,10 +408,17 @@ typedef struct {
                               /* requests are split into parts                   */
     uint32_t slot_requests;   /* request parts one batch holds (4096)            */
     uint32_t max_pending;     /* queued parts before submit refuses (2^20)       */
-    uint32_t giant_after;     /* baby steps after which a walk is handed to the  */
-                              /* warp-per-d giant-step kernel (131072); this  */
-                              /* cuts the latency of batches holding a very   */
-                              /* long period; 0xffffffff: never               */
+    uint32_t giant_after;     /* 0 (default): batches run the lane search, with  */
+                              /* the context's tuning table or the library's own */
+                              /* settings, where the batch's largest d has one,  */
+                              /* EIS_OPT_STEP_LIMIT is at its default or above   */
+                              /* and the slots' tables fit an eighth of the      */
+                              /* context's budget (about 0.7 GB a slot, charged  */
+                              /* to it); else as 131072.  n > 0: batches walk,   */
+                              /* and a walk is handed to the warp-per-d          */
+                              /* giant-step kernel after n baby steps, which     */
+                              /* cuts the latency of batches holding a very long */
+                              /* period; 0xffffffff: never                       */
     uint32_t giant_max;       /* at most this many walks per batch go to the     */
                               /* giant-step kernel (0: slot_candidates / 8)      */
     uint32_t fail_launches;   /* test hook (0): the first n batch launches fail  */
@@ -431,7 +438,8 @@ typedef struct {
     uint64_t pending_parts;
     uint64_t reserved_bytes;  /* device memory of the slots */
     uint64_t deferred;        /* walks of range parts handed to the giant-step */
-                              /* kernel after giant_after baby steps           */
+                              /* kernel after giant_after baby steps (batches  */
+                              /* that search hand none on)                     */
 } eis_server_counters;
 
 /* Start a server on ctx's device.  Device memory for `slots` batches is

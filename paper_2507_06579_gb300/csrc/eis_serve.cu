@@ -7,7 +7,9 @@
 // context budget) and pinned host tables.  Whenever a slot is free the
 // dispatcher packs as many queued request parts as fit (candidates and
 // segment count) into one batch and launches the whole pipeline -- sieve,
-// compaction, persistent walk, count -- on the slot's stream.  Requests that
+// compaction, the lane search (recording walk, search, fallback walk, in rounds)
+// or the persistent walk with its long walks handed to k_giant, count -- on the
+// slot's stream; membership queries go to k_giant.  Requests that
 // arrive while batches run queue on the host and go out in the next free
 // slot, so up to `slots` batches overlap on the device: a persistent walk
 // CTA exits as soon as its lanes run out of work, and the next batch's CTAs
@@ -238,7 +240,9 @@ bool launch_batch(eis_server *s, Slot &sl) {
         k_compact<<<nt, 256, 0, st>>>(sl.d_tiles, sl.d_sqfree, sl.d_tile_off, sl.d_surv, nullptr,
                                       nullptr, nullptr);
         const int fast = dmax < kFastDLimit ? 1 : 0;
-        const bool search = s->search_chunk && dmax >= s->tt.d_hi[0];
+        // (a batch whose largest d have no search of their own walks, and hands its
+        // long walks on)
+        const bool search = s->search_chunk && s->tt.nbaby[tune_row(s->tt, dmax)] > 0;
         if (search) {
             // at most about 0.82 of the candidates are square-free; the last
             // round takes whatever is left

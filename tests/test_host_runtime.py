@@ -183,3 +183,22 @@ def test_kept_memory_gives_way_where_the_device_has_no_more(rt):
         grown(c)
         with E.Server(c, slots=1, slot_candidates=1 << 16, giant_after=131072) as srv:  # refused before
             srv.stats()
+
+
+@pytest.mark.parametrize("rows,lo,search", [
+    ([], 10**12, True), ([], 10**6, False),
+    ([(10**9, 0, 16)], 10**12, False),   # tuned below 10^9 only: the last row covers every larger d
+    ([(10**9, 0, 16), (10**10, 512, 16)], 10**12, True),
+    ([(10**9, 512, 16), (10**10, 0, 16)], 10**12, False),
+    ([(E.EIS_D_LIMIT, 512, 16)], 10**6, True),
+])
+def test_a_servers_batch_searches_or_hands_long_walks_on(rt, rows, lo, search):
+    """As the tuning row of the batch's largest d says; a batch that walks hands
+    its long walks to the giant-step kernel."""
+    with E.Context(0) as c:
+        c.set_tune_table(rows)
+        with E.Server(c, slots=1) as srv:
+            rt.fake_reset()
+            srv.wait(srv.submit_count(lo, lo + 8000))
+            assert (rt.fake_launches(b"k_walk_record") > 0) == search
+            assert (rt.fake_launches(b"k_giant") > 0) == (not search)
