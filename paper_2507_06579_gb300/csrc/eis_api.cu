@@ -156,6 +156,8 @@ struct eis_plan {
     size_t res_bytes = 0;
     std::vector<unsigned char> res;  // host copy of the last launch's results
     bool fetched = false;
+    bool replayed = false;  // launched into a stream under capture: the caller's graph
+                            // runs the plan again without a plan_launch
 };
 
 // ------------------------------------------------------------------ helpers
@@ -916,16 +918,20 @@ static int plan_launch(eis_plan *p, cudaStream_t s) {
         int rc = plan_enqueue(p, s, false);
         if (rc != EIS_OK) return rc;
     }
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    EIS_CK(cudaStreamIsCapturing(s, &cap));
+    p->replayed |= cap != cudaStreamCaptureStatusNone;
     p->last_stream = s;
     p->launched = true;
     p->fetched = false;
     return EIS_OK;
 }
 
-// Wait for the last launch and bring its results (p->res) to the host, once.
+// Wait for the last launch and bring its results (p->res) to the host, once a
+// launch (a replayed plan's every time).
 static int plan_wait(eis_plan *p) {
     if (!p->launched) return EIS_EINVAL;
-    if (!p->fetched) {
+    if (!p->fetched || p->replayed) {
         unsigned char *pinned = p->res_bytes <= kPinnedRes ? p->ctx->h_res : nullptr;
         p->res.resize(p->res_bytes);
         EIS_CK(cudaMemcpyAsync(pinned ? pinned : p->res.data(), p->d_res, p->res_bytes,

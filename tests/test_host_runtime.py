@@ -202,3 +202,25 @@ def test_a_servers_batch_searches_or_hands_long_walks_on(rt, rows, lo, search):
             srv.wait(srv.submit_count(lo, lo + 8000))
             assert (rt.fake_launches(b"k_walk_record") > 0) == search
             assert (rt.fake_launches(b"k_giant") > 0) == (not search)
+
+
+def test_results_of_a_replayed_plan_are_fetched_again(rt):
+    """A launch's results come to the host once; those of a plan that a caller's
+    graph replays are waited for and read at every call."""
+    with E.Context(0) as c:
+        c.set_option(E.EIS_OPT_USE_GRAPH, 0)
+        p = c.plan_create([10**9], [10**9 + 8000])
+
+        def waits():
+            n = rt.fake_waits()
+            p.counts()
+            p.copy_bitmaps()
+            return rt.fake_waits() - n
+
+        p.launch(777)
+        assert waits() == 1 and waits() == 0
+        rt.fake_capture(777, 1)
+        p.launch(777)
+        rt.fake_capture(777, 0)
+        assert waits() == 2 and waits() == 2
+        p.destroy()
