@@ -23,6 +23,13 @@
 // lasts at least until it has passed one marked state and looked it up under
 // both keys; the next composition starts from wherever the walk stopped.
 //
+// The kernels' cycle.  The stride is Y = reduce(a_jl * a_j'), j' the last table
+// state at least kBsgsWideGap steps before jl (or a_jl itself).  Where two norms
+// share a factor the product (nuc_mul, eis_nuc.cuh) is not formed: the stride's
+// a_jl, and a cycle's mu, step on and try again, and Y moves on to a norm without
+// small factors.  Each cycle looks up its first marked state x and composes from
+// x + 1 (moved on as said).
+//
 // Why the first hit is in the first period.  Every marked state at position
 // l - jl .. l + jl is in the table (directly or as a mirror).  A walk that
 // starts inside that window meets a marked state before leaving it (l and
@@ -34,6 +41,12 @@
 // few dozen, so no gap can hold the whole window.  Walks only move forward
 // from position jl on, so a direct key cannot match a baby position
 // (j <= jl) in the first period.  Hence the first hit is at l - j or l + j.
+// With the wide stride a cycle that starts before the window goes at most
+//   delta_jl + delta_j' + (kStrideSteps + kCycleSteps + 1 steps) + kappa + kappa',
+// against the window's 2 delta_jl: the 64 steps between j' and jl (76 of distance
+// at 1.187 a step) are to hold 41 (49) and the two products' offsets, which are
+// below 0 (-0.1 to -22 in 2.1e5 products of states of d from 10^10 to 2^44, -7 on
+// average: a product lands short of the sum of the distances).
 #pragma once
 
 #include <cmath>
@@ -50,6 +63,10 @@ constexpr int kBsgsMinJl = 256;           // a d is searched only if its last ma
                                           // is at least this far in (window margin)
 constexpr int kBsgsWideGap = 64;          // the wide stride a_jl * a_j' takes the last
                                           // table state j' <= jl - kBsgsWideGap
+constexpr int kStrideSteps = 24;          // steps that may go into the wide stride beside
+                                          // its product, ...
+constexpr uint32_t kCycleSteps = 16;      // ... and into a cycle before its product: past
+                                          // them the fallback walk finishes the d
 constexpr uint32_t kBsgsEntryBytes = 16;
 constexpr uint32_t kBsgsRegionBytes = kBsgsKmax * kBsgsEntryBytes;  // 2048: the entries
 
@@ -119,6 +136,23 @@ EIS_HD float bsgs_num(int64_t P, int64_t s, bool fast) {
     return fast ? v + 0.5f : v;
 }
 
+// Per-lane filter of a d's table (in shared memory): kFilterWords words, in which
+// every entry sets two bits of one word, all three chosen by a hash of its Q (the
+// direct and the mirror key of a state share it).  A Q whose bits are not both
+// set is not in the table; a match is settled by an exact scan of the entries
+// (40 entries: 1 look-up in 170 scans in vain).
+constexpr int kFilterWords = 32;
+
+EIS_HD void bsgs_filter_bits(uint32_t q, uint32_t &word, uint32_t &mask) {
+    uint32_t h = q * 0x9E3779B1u;
+    h ^= h >> 15;
+    h *= 0x2C1B3C6Du;
+    word = h >> 27;
+    mask = (1u << ((h >> 22) & 31u)) | (1u << ((h >> 17) & 31u));
+}
+
+// An open-addressing index of the entries by (Q, num), for the host model of the
+// first products only.
 EIS_HD uint32_t bsgs_slot(uint32_t q, uint32_t num) {
     uint32_t h = q * 0x9E3779B1u ^ num * 0x85EBCA6Bu;
     h ^= h >> 15;

@@ -227,15 +227,37 @@ EIS_HD NucIdeal nuc_step(const NucIdeal &X, int32_t s) {
     return o;
 }
 
-// The first state from X on whose norm no prime up to 13 divides (at most 16
-// steps on): its products meet a common factor 1 time in 70, against 1 in 5.
-EIS_HD NucIdeal nuc_coprime(NucIdeal X, int32_t s) {
-    for (int i = 0; i < 16; ++i) {
+// The first state from X on whose norm no prime up to 13 divides (at most `most`
+// steps on, counted in `steps`): its products meet a common factor 1 time in 70,
+// against 1 in 5.
+EIS_HD NucIdeal nuc_coprime(NucIdeal X, int32_t s, int most, int &steps) {
+    for (int i = 0; i < most; ++i) {
         const uint32_t a = (uint32_t)X.a;
         if (a % 3 && a % 5 && a % 7 && a % 11 && a % 13) break;
         X = nuc_step(X, s);
+        ++steps;
     }
     return X;
+}
+
+// The lane search's wide stride: M = reduce(x J), x the first state from G on
+// whose norm has no factor in common with J's (few d need more than two steps;
+// one without the wide stride would take twice the giant steps), and Y the first
+// from M on without small factors.  At most kStrideSteps steps in all (`steps`):
+// they come out of the window's margin (eis_bsgs.cuh).  False: no product.
+EIS_HD bool nuc_stride(const NucIdeal &G, const NucIdeal &J, int32_t s, int32_t L, NucIdeal &M,
+                       NucIdeal &Y, int &steps) {
+    NucIdeal x = G;
+    int st = kNucRetry;
+    for (steps = 0; steps < kStrideSteps; ++steps) {
+        if (steps) x = nuc_step(x, s);
+        st = nuc_mul(x, J, s, L, M);
+        if (st != kNucRetry) break;
+    }
+    if (st != kNucOk) return false;
+    const int left = kStrideSteps - steps;
+    Y = nuc_coprime(M, s, left < 16 ? left : 16, steps);
+    return true;
 }
 
 }  // namespace eis

@@ -293,22 +293,13 @@ __global__ void __launch_bounds__(128) k_prep(const Seg *__restrict__ segs, uint
         const int32_t L = (int32_t)isqrt44((uint64_t)s);
         const NucIdeal G = entry_ideal(ge, s, d);
         NucIdeal M = G, Y = G;
-        int st = kNucRetry;
-        if (ej > 0) {
-            const NucIdeal J = entry_ideal(e[ej], s, d);
-            NucIdeal x = G;
-            // a common factor: one step on (few d need more than two; one without
-            // the wide stride would take twice the giant steps)
-            for (int t = 0; t < 24 && st == kNucRetry; ++t) {
-                if (t) x = nuc_step(x, s);
-                st = nuc_mul(x, J, s, L, M);
-            }
-            if (st == kNucOk) Y = nuc_coprime(M, s); else M = G;
-        }
+        int steps;
+        const bool wide = ej > 0 && nuc_stride(G, entry_ideal(e[ej], s, d), s, L, M, Y, steps);
+        if (!wide) M = G;
         const float T = __fmul_rn(tt.tau[tune_row(tt, (uint64_t)d)], __uint2float_rn((uint32_t)s));
         r[1] = make_uint4((uint32_t)M.a, (uint32_t)M.b, (uint32_t)M.g, (uint32_t)M.w);
         r[2] = make_uint4((uint32_t)Y.a, (uint32_t)Y.b, (uint32_t)Y.g, (uint32_t)Y.w);
-        r[3] = make_uint4(st == kNucOk, (uint32_t)L, __float_as_uint(T), 0u);
+        r[3] = make_uint4(wide, (uint32_t)L, __float_as_uint(T), 0u);
     }
 }
 
@@ -326,27 +317,12 @@ __device__ __forceinline__ void fallback(uint32_t *fb_list, uint32_t *fb_count, 
         atomicOr(status, kErrGiant);
 }
 
-// Per-lane filter of a d's table in shared memory: 32 words, in which every
-// entry sets two bits of one word, all three chosen by a hash of its Q (the
-// direct and the mirror key of a state share it).  A Q whose bits are not both
-// set is not in the table; a match is settled by an exact scan of the entries
-// (40 entries: 1 look-up in 170 scans in vain).
-// An entry costs one hash and one shared atomic, all 32 lanes at once.  The
-// open-addressing index of 8-bit fingerprints it replaces cost about 40,000
+// The filter's entry costs one hash and one shared atomic, all 32 lanes at once.
+// The open-addressing index of 8-bit fingerprints it replaces cost about 40,000
 // issue slots a d (probe loops and compare-and-swap retries), two thirds of the
 // search once k_cubic has left only short periods: 18.6 -> 14.4 ms for the
 // window's 1.2e7 d at N = 768, m = 24.  128 B a lane also lets 8 blocks
 // reside instead of 6.
-constexpr int kFpWords = 32;
-
-__device__ __forceinline__ void fp_bits(uint32_t q, uint32_t &word, uint32_t &mask) {
-    uint32_t h = q * 0x9E3779B1u;
-    h ^= h >> 15;
-    h *= 0x2C1B3C6Du;
-    word = h >> 27;
-    mask = (1u << ((h >> 22) & 31u)) | (1u << ((h >> 17) & 31u));
-}
-
 struct SIdeal {
     int32_t a, b, g;
 };
@@ -364,8 +340,8 @@ __device__ __forceinline__ void bsgs_body(
     const uint32_t pause = min(groups, (walk_pause + kBsgsGroup - 1) / kBsgsGroup);
     const int lane = threadIdx.x & 31;
     const unsigned lt = lanemask_lt();
-    uint32_t *fp_warp = fp_all + (threadIdx.x & ~31u) * kFpWords;  // lane t's words at t * kFpWords
-    uint32_t *fp_mine = fp_warp + lane * kFpWords;
+    uint32_t *fp_warp = fp_all + (threadIdx.x & ~31u) * kFilterWords;  // lane t's words at t * kFilterWords
+    uint32_t *fp_mine = fp_warp + lane * kFilterWords;
     bool active = false, exhausted = false;
     uint32_t cand = 0, cycles = 0, k = 0;
     int64_t d = 0;
@@ -412,6 +388,7 @@ __device__ __forceinline__ void bsgs_body(
                     landed = r3.x != 0;  // its first product is taken: walk on from it
                     compose_now = !landed;
                     cycles = landed;
+                    walked = 0;
                     L = (int32_t)r3.y;
                     T = __uint_as_float(r3.z);
                     C = __uint2float_rn((uint32_t)(kFast ? 2 * s + 1 : 2 * s));
@@ -429,7 +406,7 @@ __device__ __forceinline__ void bsgs_body(
             const uint32_t kk = __shfl_sync(kFull, k, src);
             const uint4 *e = reinterpret_cast<const uint4 *>(
                 __shfl_sync(kFull, reinterpret_cast<unsigned long long>(tab), src));
-            uint32_t *sl = fp_warp + src * kFpWords;
+            uint32_t *sl = fp_warp + src * kFilterWords;
             uint32_t q[kBsgsKmax / 32];  // (all loads in flight at once)
 #pragma unroll
             for (int t = 0; t < kBsgsKmax / 32; ++t)
@@ -440,7 +417,7 @@ __device__ __forceinline__ void bsgs_body(
             for (int t = 0; t < kBsgsKmax / 32; ++t)
                 if (lane + 32 * t < kk) {
                     uint32_t word, mask;
-                    fp_bits(q[t], word, mask);
+                    bsgs_filter_bits(q[t], word, mask);
                     atomicOr(&sl[word], mask);
                 }
             __syncwarp();
@@ -466,12 +443,14 @@ __device__ __forceinline__ void bsgs_body(
                 nx = NucIdeal{(int32_t)o.a, (int32_t)o.b, o.g, (int32_t)(-Qm / 2)};
             }
             if (++cycles > max_cycles) st = kNucFail;
+            if (st == kNucRetry && ++walked > kCycleSteps) st = kNucFail;
             if (st == kNucFail) {
                 fallback(fb_list, fb_count, fb_cap, cand, status);
                 my_cycles += cycles;
                 active = false;
             } else if (st == kNucRetry) {
-                // the norms share a factor: one step on, next iteration again
+                // the norms share a factor: one step on, next iteration again (`walked`
+                // counts these while the lane composes)
                 const NucIdeal m1 = nuc_step(NucIdeal{mu.a, mu.b, mu.g, wmu}, s);
                 mu = SIdeal{m1.a, m1.b, m1.g};
                 wmu = m1.w;
@@ -520,6 +499,7 @@ __device__ __forceinline__ void bsgs_body(
             gc += (int)walked + 1 + w.x;
             ++my_walk;
             compose_now = true;
+            walked = 0;
         }
         if (active && !compose_now && walked >= walk_cap) {
             // no marked state within walk_cap steps: the fallback walk finishes it
@@ -534,7 +514,7 @@ __device__ __forceinline__ void bsgs_body(
         const uint32_t kq = __float_as_uint(w.Qp), kd = __float_as_uint(numx),
                        km = __float_as_uint(w.num);
         uint32_t fword, fmask;
-        fp_bits(kq, fword, fmask);
+        bsgs_filter_bits(kq, fword, fmask);
         const bool maybe = at_end && (fp_mine[fword] & fmask) == fmask;
         int g = -1;
         // exact scan of the tables of the lanes with a match, by
@@ -597,7 +577,7 @@ __global__ void __launch_bounds__(128, kCompose == 0 ? 8 : 1) k_bsgs_t(
     unsigned long long *__restrict__ acc, int *__restrict__ status, uint32_t *__restrict__ fb_list,
     uint32_t *__restrict__ fb_count, uint32_t fb_cap, const __grid_constant__ TuneTab tt,
     uint32_t max_cycles, uint32_t walk_cap, uint32_t walk_window, uint32_t walk_pause) {
-    __shared__ uint32_t fp_all[128 * kFpWords];
+    __shared__ uint32_t fp_all[128 * kFilterWords];
     bsgs_body<kFast, kCompose>(segs, nseg, recs, nrec, rec_cap, next_ptr, pool, flags, glog, acc,
                                status, fb_list, fb_count, fb_cap, tt, max_cycles, walk_cap,
                                walk_window, walk_pause, fp_all);

@@ -56,7 +56,8 @@ __device__ __noinline__ int4 query_mul(int4 X, int4 Y, int64_t d, int32_t s, int
             return make_int4(0, 0, 0, 0);
         out = NucIdeal{(int32_t)o.a, (int32_t)o.b, o.g, (int32_t)(-Qm / 2)};
     }
-    out = nuc_coprime(out, s);
+    int steps = 0;
+    out = nuc_coprime(out, s, 16, steps);
     return make_int4(out.a, out.b, out.g, out.w);
 }
 
