@@ -44,7 +44,7 @@
 // With the wide stride a cycle that starts before the window goes at most
 //   delta_jl + delta_j' + (kStrideSteps + kCycleSteps + 1 steps) + kappa + kappa',
 // against the window's 2 delta_jl: the 64 steps between j' and jl (76 of distance
-// at 1.187 a step) are to hold 41 (49) and the two products' offsets, which are
+// at 1.187 a step) are to hold 57 (68) and the two products' offsets, which are
 // below 0 (-0.1 to -22 in 2.1e5 products of states of d from 10^10 to 2^44, -7 on
 // average: a product lands short of the sum of the distances).
 #pragma once
@@ -65,8 +65,11 @@ constexpr int kBsgsWideGap = 64;          // the wide stride a_jl * a_j' takes t
                                           // table state j' <= jl - kBsgsWideGap
 constexpr int kStrideSteps = 24;          // steps that may go into the wide stride beside
                                           // its product, ...
-constexpr uint32_t kCycleSteps = 16;      // ... and into a cycle before its product: past
+constexpr uint32_t kCycleSteps = 32;      // ... and into a cycle before its product: past
                                           // them the fallback walk finishes the d
+                                          // (below 2^44 1 d in 10^5 takes 17 in one of its
+                                          // hundreds of cycles, where Y kept a small
+                                          // factor; each further one is 0.6 times as rare)
 constexpr uint32_t kBsgsEntryBytes = 16;
 constexpr uint32_t kBsgsRegionBytes = kBsgsKmax * kBsgsEntryBytes;  // 2048: the entries
 

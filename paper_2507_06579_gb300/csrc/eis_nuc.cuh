@@ -255,8 +255,7 @@ EIS_HD bool nuc_stride(const NucIdeal &G, const NucIdeal &J, int32_t s, int32_t 
         if (st != kNucRetry) break;
     }
     if (st != kNucOk) return false;
-    const int left = kStrideSteps - steps;
-    Y = nuc_coprime(M, s, left < 16 ? left : 16, steps);
+    Y = nuc_coprime(M, s, kStrideSteps - steps, steps);
     return true;
 }
 

@@ -51,7 +51,7 @@ def test_every_hit_is_in_the_first_period(stride_host, orc, lo, hi, n, settings,
     searched = 0
     for (d, N, m, _), (status, g, cycles, steps, stride, filtered, hit) in zip(rows, _run(stride_host, rows)):
         assert status in (0, 1, 2), (d, N, m, status)
-        assert filtered == 0 and steps <= 16 and stride <= 24
+        assert filtered == 0 and steps <= 32 and stride <= 24
         if status < 2:
             rc, theta, _ = orc.walk_mod2(d)
             assert rc == 0 and g == theta - 1, (d, N, m)
