@@ -473,8 +473,8 @@ def main():
                                "[1e6, 1e12], L log-uniform in [1e2, 1e6]; 10% membership "
                                "queries on d == 5 mod 8 below 1e12 (not-square-free d answer "
                                "EIS_ENOTD); seed 5",
-                   "server": "4 slots x 2^22 candidates, continuous batching; walks past "
-                             "131072 baby steps and membership queries go to the warp-per-d "
+                   "server": "4 slots x 2^22 candidates, continuous batching; batches run "
+                             "the lane search, membership queries go to the warp-per-d "
                              "giant-step kernel",
                    "rates": rates,
                    "saturation": ({"offered_rps": sat["rate_rps"],
@@ -585,8 +585,9 @@ def main():
                 "dtype": "int (exact; < 2^23 in fp32 registers)",
                 "dtype_note": "every value is an integer (or integer + 1/2) below 2^23, "
                               "carried exactly in fp32 registers with exact adds, "
-                              "multiply-adds and a directed-rounding quotient; sieve, set-up "
-                              "and giant steps in u64/i64; results are bit-exact integers",
+                              "multiply-adds and a directed-rounding quotient; sieve and "
+                              "set-up in u64/i64, giant steps in 32-bit integers and exact "
+                              "fp32; results are bit-exact integers",
                 "data": "synthetic",
                 "config": {"workload": "all square-free d == 5 mod 8 in [1e11-%.0e, 1e11] "
                                        "(per rank: its own window below 1e11)" % args.window,
