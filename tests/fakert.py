@@ -20,11 +20,15 @@ def load():
     global _fake
     if _fake is None:
         E.build()
+        objs = sorted(glob.glob(os.path.join(_build.BUILD, "*.cu.o")))
+        if len(objs) < len(_build.sources()):  # the library without its objects
+            E.build(force=True)
+            objs = sorted(glob.glob(os.path.join(_build.BUILD, "*.cu.o")))
         inc = os.path.join(os.path.dirname(os.path.dirname(_build.nvcc())), "include")
         out = os.path.join(tempfile.mkdtemp(), "libeis_fake.so")
         subprocess.run(["g++", "-std=c++17", "-O1", "-shared", "-fPIC", "-Wl,-Bsymbolic", "-I", inc,
                         os.path.join(ROOT, "tests", "fake_cudart.cpp"),
-                        *sorted(glob.glob(os.path.join(_build.BUILD, "*.cu.o"))),
+                        *objs,
                         "-o", out, "-ldl", "-lpthread"], check=True)
         L = ctypes.CDLL(out)
         for name, res, args in E.SIGNATURES:
